@@ -21,6 +21,8 @@ struct d3m_ctx {
   Symbolic S;
   d3m_options opt{};
   bool fp64 = true, tc = false, tf32 = false;
+  bool dig = false;                  // FP64 unpivoted: tile products as exact digit products (factor_dig.cu)
+  bool resid = true;                 // the residual's buffers and digit planes exist
   int b = 64;
   int device = 0, nsm = 0;
   size_t csize = 16;                 // bytes of one factor element
@@ -64,6 +66,8 @@ struct d3m_ctx {
   void* opA = nullptr;
   void* opB = nullptr;
   void* opS = nullptr;               // TF32: bf16 split planes of L for the solve's tensor-core products
+  int32_t* expA = nullptr;           // digit engine: row scales of opA / opB
+  int32_t* expB = nullptr;
   void* Sacc = nullptr;
   void* E = nullptr;                 // pivot mode: sub-diagonals of the 2 x 2 pivot blocks [NT][b]
   int32_t* piv = nullptr;            // pivot mode: permutation of every diagonal tile [NT][b]
@@ -548,8 +552,9 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
   h->L = dalloc<unsigned char>(h, (size_t)ntiles * b * b * h->csize);
   h->Linv = dalloc<unsigned char>(h, (size_t)S.NT * b * b * h->csize);
   h->D = dalloc<unsigned char>(h, (size_t)S.NT * b * h->csize);
-  h->Sacc = dalloc<unsigned char>(h, (size_t)std::max<int64_t>(1, S.n_acc) * b * b * h->csize);
-  if (!h->L || !h->Linv || !h->D || !h->Sacc) return set_err(h, D3M_ERR_OOM, "cudaMalloc failed for the factor tiles");
+  // the SIMT and FP64 engines accumulate a tile's updates where its L ends up
+  if (h->tc) h->Sacc = dalloc<unsigned char>(h, (size_t)std::max<int64_t>(1, S.n_acc) * b * b * h->csize);
+  if (!h->L || !h->Linv || !h->D || (h->tc && !h->Sacc)) return set_err(h, D3M_ERR_OOM, "cudaMalloc failed for the factor tiles");
   if (h->opt.pivot) {
     h->E = dalloc<unsigned char>(h, (size_t)S.NT * b * h->csize);
     h->piv = dalloc<int32_t>(h, (size_t)S.NT * b);
@@ -734,14 +739,18 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
     const int ngrp = resid_tc_groups(mr, &nr_grp);   // the most groups any nrhs <= max_nrhs uses
     r.xs_total = pb;
     r.nblk = S.N;
-    ALLOC(r.kdig, unsigned short, pa * 128 * 32);
-    ALLOC(r.xdig, unsigned short, pb * ngrp * 64 * 32);
-    ALLOC(r.Kmax_bits, unsigned long long, S.nnzb_K);
-    ALLOC(r.Kdiag, double2, S.n);
-    ALLOC(r.rowsum, float, S.n);
-    ALLOC(r.xT, int, (size_t)ngrp * S.N * 32);
-    std::string e3;
-    if (resid_tc_make_maps(r.kdig, pa, r.xdig, pb * ngrp, &h->rtc_maps, e3) != 0) return set_err(h, D3M_ERR_CUDA, e3);
+    // an FP64 solve without omega never forms a residual
+    h->resid = !h->fp64 || h->opt.fp64_omega != 0;
+    if (h->resid) {
+      ALLOC(r.kdig, unsigned short, pa * 128 * 32);
+      ALLOC(r.xdig, unsigned short, pb * ngrp * 64 * 32);
+      ALLOC(r.Kmax_bits, unsigned long long, S.nnzb_K);
+      ALLOC(r.Kdiag, double2, S.n);
+      ALLOC(r.rowsum, float, S.n);
+      ALLOC(r.xT, int, (size_t)ngrp * S.N * 32);
+      std::string e3;
+      if (resid_tc_make_maps(r.kdig, pa, r.xdig, pb * ngrp, &h->rtc_maps, e3) != 0) return set_err(h, D3M_ERR_CUDA, e3);
+    }
   }
   UPLOAD(h->m_orig, S.m_orig);
   UPLOAD(h->xoff_orig, S.xoff_orig);
@@ -776,6 +785,35 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
   CUDA_TRY(h, cudaMemset(h->sweep_status, 0, sizeof(int)));
   ALLOC(h->contract, double2, S.N);
   CUDA_TRY(h, cudaMallocHost(&h->h_stat, 3 * sizeof(double)));
+  // FP64 without pivoting: the digit engine, where its words (16 bytes per complex entry of L and of
+  // W, beside L itself) leave a quarter of the free memory to the caller; else the SIMT engine,
+  // which needs none of them
+  if (h->fp64 && !h->opt.pivot) {
+    const size_t words = (size_t)ntiles * 2 * b * b * sizeof(unsigned long long), exps = (size_t)ntiles * b;
+    size_t mfree = 0, mtotal = 0;
+    if (cudaMemGetInfo(&mfree, &mtotal) != cudaSuccess) cudaGetLastError();
+    int32_t most = 0;                  // the engine lists a task's products in shared memory
+    for (const TileTask& t : S.tasks) most = std::max(most, t.nk);
+    if (most <= kDigMaxProducts && 2 * words <= mfree / 4 * 3) {
+      h->opA = dalloc<unsigned char>(h, words);
+      h->opB = dalloc<unsigned char>(h, words);
+      h->expA = dalloc<int32_t>(h, exps);
+      h->expB = dalloc<int32_t>(h, exps);
+      h->dig = h->opA && h->opB && h->expA && h->expB;
+      if (!h->dig) {
+        void* part[4] = {h->opA, h->opB, h->expA, h->expB};
+        const size_t bytes[4] = {words, words, exps * sizeof(int32_t), exps * sizeof(int32_t)};
+        for (int q = 0; q < 4; ++q)
+          if (part[q]) {
+            h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), part[q]));
+            h->dev_bytes -= (int64_t)bytes[q];
+            cudaFree(part[q]);
+          }
+        h->opA = h->opB = nullptr;
+        h->expA = h->expB = nullptr;
+      }
+    }
+  }
 #undef ALLOC
 #undef UPLOAD
   return D3M_OK;
@@ -932,6 +970,8 @@ static int enqueue_factor(d3m_ctx* h, const void* Kin, bool kdev, cudaStream_t s
   p.opA = h->opA;
   p.opB = h->opB;
   p.opS = h->opS;
+  p.expA = h->expA;
+  p.expB = h->expB;
   p.k_arrived = kup ? h->k_arrived : nullptr;
   p.Sacc = h->Sacc;
   p.trace = h->trace;
@@ -943,6 +983,7 @@ static int enqueue_factor(d3m_ctx* h, const void* Kin, bool kdev, cudaStream_t s
   if (h->trace) CUDA_TRY(h, cudaMemsetAsync(h->trace, 0xff, (size_t)10 * ntiles * sizeof(int64_t), st));
   ev_begin(h, d3m_ctx::EV_FACTOR, st);
   if (h->tc) rc = launch_factor_tc(p, h->maps, h->tf32, h->nsm, st);
+  else if (h->dig) rc = launch_factor_dig(p, h->nsm, st);
   else rc = launch_factor_simt(p, h->fp64, h->nsm, st);
   if (rc) return set_err(h, D3M_ERR_CUDA, std::string("factor launch: ") + cudaGetErrorString((cudaError_t)rc));
   ev_end(h, d3m_ctx::EV_FACTOR, st);
@@ -951,23 +992,23 @@ static int enqueue_factor(d3m_ctx* h, const void* Kin, bool kdev, cudaStream_t s
   // ||K_i||_inf and the digit planes of K (for the residual) on a second stream, concurrently
   // with the block inverses: the persistent factorization holds every SM, the smaller kernels
   // share them
-  CUDA_TRY(h, cudaEventRecord(h->ev_fork, st));
-  CUDA_TRY(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
-  {
+  if (h->resid) {
+    CUDA_TRY(h, cudaEventRecord(h->ev_fork, st));
+    CUDA_TRY(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
     ResidualTc rp = resid_params(h, Ksrc);
     CUDA_TRY(h, cudaMemsetAsync(rp.kmax, 0, h->ninst * sizeof(unsigned), h->side));
     rc = launch_kdigits(rp, (int)S.nnzb_K, (int)S.res_blk.size(), h->max_rtiles, S.N, h->side);
     if (rc) return set_err(h, D3M_ERR_CUDA, std::string("K digit launch: ") + cudaGetErrorString((cudaError_t)rc));
     h->launches += 3;
+    CUDA_TRY(h, cudaEventRecord(h->ev_join, h->side));
   }
-  CUDA_TRY(h, cudaEventRecord(h->ev_join, h->side));
   if (h->use_inv && h->n_inv_work > 0) {
     rc = launch_inv_build(h->inv_work, h->n_inv_work, h->tstart, h->tcolptr, h->inv_off, h->invT_off, h->L, h->Linv,
                           h->Inv, h->InvT, h->b, st);
     if (rc) return set_err(h, D3M_ERR_CUDA, std::string("block inverse launch: ") + cudaGetErrorString((cudaError_t)rc));
     h->launches += 1;
   }
-  CUDA_TRY(h, cudaStreamWaitEvent(st, h->ev_join, 0));
+  if (h->resid) CUDA_TRY(h, cudaStreamWaitEvent(st, h->ev_join, 0));
   CUDA_TRY(h, cudaMemcpyAsync(h->h_ctl, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
   return D3M_OK;
 }

@@ -46,11 +46,13 @@ struct FactorParams {
   void* L;               // [ntiles][b][b] complex (row-major tiles)
   void* Linv;            // [NT][b][b] inverse of the unit-lower diagonal tiles
   void* D;               // [NT][b] pivots
-  void* opA;             // tensor-core operand planes (bf16) of L tiles
-  void* opB;             // tensor-core operand planes (bf16) of W tiles / T_J
+  void* opA;             // tensor-core operand planes (bf16) of L tiles; FP64: digit words of L / X_JJ
+  void* opB;             // tensor-core operand planes (bf16) of W tiles / T_J; FP64: digit words of W
+  int32_t* expA;         // FP64 digit engine: row scales of opA, opB [ntiles][b]
+  int32_t* expB;
   void* opS;             // TF32 engine: bf16 split planes of the L tiles for the solve's products, or nullptr
   const int32_t* k_arrived;  // upload progress of a host K (stored blocks in upload order), or nullptr
-  void* Sacc;            // [n_acc][b][b] partial Schur accumulators (complex, working precision)
+  void* Sacc;            // [n_acc][b][b] partial Schur accumulators (tensor-core c64 engines; the others use L's tiles)
   int64_t* trace;        // [ntasks][8] task records, or nullptr
   int64_t timeout_ns;
   double piv_tol;        // breakdown: |d| < piv_tol * max|S| of the diagonal tile

@@ -1,7 +1,7 @@
 // Persistent block-DAG factorization with a SIMT tile engine (tile edge 64).
 //
-// R = double: the plain FP64 (complex128) path; R = float: complex64 factors without tensor
-// cores (used as the SIMT reference of the mixed path).
+// R = double: FP64 (complex128) with pivoting, or where the digit engine's words (factor_dig.cu) do not
+// fit; R = float: complex64 factors without tensor cores (the SIMT engine of the mixed path).
 //
 // Each task works on one lower tile (I, J) of L (paper Sec. II: per nonzero block a task doing
 // the dense update, the dense triangular solve and the dense factorization):
@@ -267,7 +267,6 @@ __global__ void __launch_bounds__(NTHR, 1) factor_simt_kernel(FactorParams p) {
   C* Lg = reinterpret_cast<C*>(p.L);
   C* Linv = reinterpret_cast<C*>(p.Linv);
   C* Dg = reinterpret_cast<C*>(p.D);
-  C* Sacc = reinterpret_cast<C*>(p.Sacc);
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
 
@@ -314,7 +313,8 @@ __global__ void __launch_bounds__(NTHR, 1) factor_simt_kernel(FactorParams p) {
       }
     }
     __syncthreads();
-    C* Sa = (T.sidx >= 0) ? Sacc + (int64_t)T.sidx * TB * TB : nullptr;
+    // the tile's accumulator lies where L_IJ ends up: its last reader, the final task, overwrites it
+    C* Sa = Lg + (int64_t)T.tile * TB * TB;
     if (T.flags & TF_UPDATE) {
       // partial update: accumulator <- S_in - sum over this segment
       C kin[4][4];

@@ -122,6 +122,9 @@ struct TcMaps {
   alignas(64) unsigned char b[128];
 };
 
+// FP64 (unpivoted) with the tile products as exact digit products on the tensor cores
+constexpr int kDigMaxProducts = 64;    // most tile products of one task
+int launch_factor_dig(const FactorParams& p, int nblocks, cudaStream_t st);
 int launch_factor_simt(const FactorParams& p, bool fp64, int nblocks, cudaStream_t st);
 // tf32 = false: bf16 planes of the split-BF16x3 engine; true: tf32 planes
 int tc_make_maps(void* opA, void* opB, int64_t ntiles, bool tf32, TcMaps* out, std::string& err);
