@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "device.cuh"
 #include "kernels.h"
@@ -150,10 +151,10 @@ __device__ __forceinline__ C shfl_xor_c(C v, int o) {
   return v;
 }
 
-template <typename C>
+template <int RC, typename C>
 __device__ __forceinline__ void quad_reduce(C* acc) {
 #pragma unroll
-  for (int j = 0; j < RCMAX; ++j)
+  for (int j = 0; j < RC; ++j)
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1) {
       acc[j].x += __shfl_xor_sync(0xffffffffu, acc[j].x, o);
@@ -161,32 +162,57 @@ __device__ __forceinline__ void quad_reduce(C* acc) {
     }
 }
 
+// Sum N values over the 16 lanes of a row group.  While more than one value is left a lane keeps the half
+// that the offset's bit of its number selects, then the last one is summed by all; lane l (of 16)
+// ends with values max(1, N / 16) (l / max(1, 16 / N)) ...  The sums are formed over the same pairs of
+// lanes for every N.
+template <int N, int O = 8, typename C>
+__device__ __forceinline__ void lane_scatter(C* f, int lane) {
+  if constexpr (O >= 1) {
+    if constexpr (N > 1) {
+      const bool up = (lane & O) != 0;
+#pragma unroll
+      for (int q = 0; q < N / 2; ++q) {
+        const C lo = f[q], hi = f[q + N / 2];
+        const C send = up ? lo : hi;
+        C keep = up ? hi : lo;
+        keep = cadd(keep, shfl_xor_c(send, O));
+        f[q] = keep;
+      }
+      lane_scatter<N / 2, O / 2>(f, lane);
+    } else {
+      f[0] = cadd(f[0], shfl_xor_c(f[0], O));
+      lane_scatter<1, O / 2>(f, lane);
+    }
+  }
+}
+
 // dst[r][j] (=, +=, or -= by MODE 0 / 1 / 2) sum_c M[r][c] V[c][j] for the 64 rows of a staged
 // half tile M ([64][ldl]); V element (c, j) at V[c * ldv + j]; dst element (r, j) at dst[r * ldd + j].
-template <typename R, int MODE>
+template <typename R, int MODE, int RC>
 __device__ __forceinline__ void rows_matvec(const typename CT<R>::C* M, int ldl, int b, const typename CT<R>::C* V,
                                             int ldv, int rc, typename CT<R>::C* dst, int ldd) {
   using C = typename CT<R>::C;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = warp * 8 + (lane >> 2), cq = lane & 3;
-  C acc[RCMAX];
+  C acc[RC];
 #pragma unroll
-  for (int j = 0; j < RCMAX; ++j) acc[j] = CT<R>::make(0, 0);
+  for (int j = 0; j < RC; ++j) acc[j] = CT<R>::make(0, 0);
   const C* mrow = M + r * ldl;
 #pragma unroll 4
   for (int c = cq; c < b; c += 4) {
     const C m = mrow[c];
     const C* v = V + c * ldv;
-    C vv[RCMAX];
+    C vv[RC];
 #pragma unroll
-    for (int j = 0; j < RCMAX; ++j) vv[j] = (j < rc) ? v[j] : CT<R>::make(0, 0);
+    for (int j = 0; j < RC; ++j) vv[j] = (j < rc) ? v[j] : CT<R>::make(0, 0);
 #pragma unroll
-    for (int j = 0; j < RCMAX; ++j) acc[j] = cfma(m, vv[j], acc[j]);
+    for (int j = 0; j < RC; ++j) acc[j] = cfma(m, vv[j], acc[j]);
   }
-  quad_reduce(acc);
+  quad_reduce<RC>(acc);
   if (cq == 0) {
 #pragma unroll
-    for (int j = 0; j < RCMAX; ++j)
+    for (int j = 0; j < RC; ++j)
       if (j < rc)
         dst[r * ldd + j] = MODE == 0 ? acc[j] : (MODE == 1 ? cadd(dst[r * ldd + j], acc[j]) : csub(dst[r * ldd + j], acc[j]));
   }
@@ -195,7 +221,7 @@ __device__ __forceinline__ void rows_matvec(const typename CT<R>::C* M, int ldl,
 // rows_matvec on a dense [64][b] strip (one bulk copy): the 4 column classes of each of a warp's 8
 // rows start at columns rotated by 4 per row, so every warp-wide load touches 32 consecutive
 // columns (no bank conflicts); b is a power of two.
-template <typename R, int MODE>
+template <typename R, int MODE, int RC>
 __device__ __forceinline__ void rows_matvec_dense(const typename CT<R>::C* M, int b, const typename CT<R>::C* V,
                                                   int ldv, int rc, typename CT<R>::C* dst, int ldd) {
   // warp w, lane l: rows rg + 16 a (rg = 2 w + l / 16, a < 4), columns l % 16 + 16 k, all right-hand
@@ -204,40 +230,32 @@ __device__ __forceinline__ void rows_matvec_dense(const typename CT<R>::C* M, in
   using C = typename CT<R>::C;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rg = 2 * warp + (lane >> 4), cg = lane & 15;
-  C acc[4][RCMAX];
+  C acc[4][RC];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int j = 0; j < RCMAX; ++j) acc[a][j] = CT<R>::make(0, 0);
+    for (int j = 0; j < RC; ++j) acc[a][j] = CT<R>::make(0, 0);
 #pragma unroll 2
   for (int c = cg; c < b; c += 16) {
-    C v[RCMAX];
+    C v[RC];
 #pragma unroll
-    for (int j = 0; j < RCMAX; ++j) v[j] = (j < rc) ? V[c * ldv + j] : CT<R>::make(0, 0);
+    for (int j = 0; j < RC; ++j) v[j] = (j < rc) ? V[c * ldv + j] : CT<R>::make(0, 0);
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
       const C m = M[(rg + 16 * a) * b + c];
 #pragma unroll
-      for (int j = 0; j < RCMAX; ++j) acc[a][j] = cfma(m, v[j], acc[a][j]);
+      for (int j = 0; j < RC; ++j) acc[a][j] = cfma(m, v[j], acc[a][j]);
     }
   }
+  // values a * RC + j: halved at every offset while more than one is left, then summed in full (the
+  // same pairs of lanes either way)
+  constexpr int NV = 4 * RC, NL = NV > 16 ? NV / 16 : 1, REP = NV < 16 ? 16 / NV : 1;
   C* f = &acc[0][0];
+  lane_scatter<NV>(f, lane);
 #pragma unroll
-  for (int o = 8, n = 32; o >= 1; o >>= 1, n >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int q = 0; q < n / 2; ++q) {
-      const C lo = f[q], hi = f[q + n / 2];
-      const C send = up ? lo : hi;
-      C keep = up ? hi : lo;
-      keep = cadd(keep, shfl_xor_c(send, o));
-      f[q] = keep;
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int q = 2 * cg + u, a = q >> 3, j = q & 7;
-    if (j < rc) {
+  for (int u = 0; u < NL; ++u) {
+    const int q = NL * (cg / REP) + u, a = q / RC, j = q % RC;
+    if (j < rc && cg % REP == 0) {
       C* d = dst + (rg + 16 * a) * ldd + j;
       *d = MODE == 0 ? f[u] : (MODE == 1 ? cadd(*d, f[u]) : csub(*d, f[u]));
     }
@@ -246,7 +264,7 @@ __device__ __forceinline__ void rows_matvec_dense(const typename CT<R>::C* M, in
 
 // dst[c][j] (=, +=, or -= by MODE 0 / 1 / 2) sum_{r < 64} M[r][c] V[r][j] for all b columns
 // of a staged half tile.
-template <typename R, int MODE>
+template <typename R, int MODE, int RC>
 __device__ __forceinline__ void cols_matvec(const typename CT<R>::C* M, int ldl, int b, const typename CT<R>::C* V,
                                             int ldv, int rc, typename CT<R>::C* dst, int ldd) {
   using C = typename CT<R>::C;
@@ -254,23 +272,23 @@ __device__ __forceinline__ void cols_matvec(const typename CT<R>::C* M, int ldl,
   const int rq = lane & 3;
   for (int c0 = 0; c0 < b; c0 += 64) {
     const int c = c0 + warp * 8 + (lane >> 2);
-    C acc[RCMAX];
+    C acc[RC];
 #pragma unroll
-    for (int j = 0; j < RCMAX; ++j) acc[j] = CT<R>::make(0, 0);
+    for (int j = 0; j < RC; ++j) acc[j] = CT<R>::make(0, 0);
 #pragma unroll 4
     for (int r = rq; r < HR; r += 4) {
       const C m = M[r * ldl + c];
       const C* v = V + r * ldv;
-      C vv[RCMAX];
+      C vv[RC];
 #pragma unroll
-      for (int j = 0; j < RCMAX; ++j) vv[j] = (j < rc) ? v[j] : CT<R>::make(0, 0);
+      for (int j = 0; j < RC; ++j) vv[j] = (j < rc) ? v[j] : CT<R>::make(0, 0);
 #pragma unroll
-      for (int j = 0; j < RCMAX; ++j) acc[j] = cfma(m, vv[j], acc[j]);
+      for (int j = 0; j < RC; ++j) acc[j] = cfma(m, vv[j], acc[j]);
     }
-    quad_reduce(acc);
+    quad_reduce<RC>(acc);
     if (rq == 0) {
 #pragma unroll
-      for (int j = 0; j < RCMAX; ++j)
+      for (int j = 0; j < RC; ++j)
         if (j < rc)
           dst[c * ldd + j] = MODE == 0 ? acc[j] : (MODE == 1 ? cadd(dst[c * ldd + j], acc[j]) : csub(dst[c * ldd + j], acc[j]));
     }
@@ -349,7 +367,7 @@ __device__ __forceinline__ void stage_rows_only(C* sV, int ldv, const C* Y, int6
         : "memory");
 }
 
-template <typename R, bool FWD>
+template <typename R, bool FWD, int RC>
 __global__ void __launch_bounds__(GGT, 1) gather_kernel(const SolveGroup* __restrict__ groups,
                                                         const SolveItem* __restrict__ items,
                                                         const typename CT<R>::C* __restrict__ L,
@@ -361,12 +379,12 @@ __global__ void __launch_bounds__(GGT, 1) gather_kernel(const SolveGroup* __rest
   const int nh = b / HR;
   const int vlen = FWD ? b : HR;                         // source rows per right-hand side
   const int ldv = vlen + (int)(16 / sizeof(C));
-  const int stg = HR * b + RCMAX * ldv;                  // elements of one stage buffer
+  const int stg = HR * b + RC * ldv;                  // elements of one stage buffer
   C* const sbase = reinterpret_cast<C*>(smem_raw);
   __shared__ __align__(8) uint64_t bars[GMAXSTG];
   __shared__ GatherMeta s_meta[GMAXSTG];
-  const int j0 = blockIdx.y * RCMAX;
-  const int rc = min(RCMAX, nrhs - j0);
+  const int j0 = blockIdx.y * RC;
+  const int rc = min(RC, nrhs - j0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   auto skip = [&](int u) {                               // first active unit >= u (whole warps)
     if (!mk.done) return u;
@@ -389,9 +407,9 @@ __global__ void __launch_bounds__(GGT, 1) gather_kernel(const SolveGroup* __rest
     for (int i = 0; i < nstg; ++i) mbar_init_s(&bars[i]);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // source rows past rc stay zero in every stage (the products run over all RCMAX rows)
-  for (int i = threadIdx.x; i < nstg * (RCMAX - rc) * ldv; i += GGT) {
-    const int st = i / ((RCMAX - rc) * ldv), e = i % ((RCMAX - rc) * ldv);
+  // source rows past rc stay zero in every stage (the products run over all RC rows)
+  for (int i = threadIdx.x; i < nstg * (RC - rc) * ldv; i += GGT) {
+    const int st = i / ((RC - rc) * ldv), e = i % ((RC - rc) * ldv);
     sbase[(int64_t)st * stg + HR * b + rc * ldv + e] = CT<R>::make(0, 0);
   }
   __syncthreads();
@@ -445,11 +463,11 @@ __global__ void __launch_bounds__(GGT, 1) gather_kernel(const SolveGroup* __rest
   // backward: warp w -> rows 8 (w % 8) .. + 7 of the half and column half w / 8, lane l -> columns
   //   l + 32 k of that half; the 8 row groups are summed through shared memory in a fixed order
   constexpr int NA = 2;                                  // rows (forward) / column slots (backward) per thread
-  C acc[NA][RCMAX];
+  C acc[NA][RC];
 #pragma unroll
   for (int a = 0; a < NA; ++a)
 #pragma unroll
-    for (int j = 0; j < RCMAX; ++j) acc[a][j] = CT<R>::make(0, 0);
+    for (int j = 0; j < RC; ++j) acc[a][j] = CT<R>::make(0, 0);
   const uint64_t deadline = globaltimer_ns() + SWEEP_TIMEOUT_NS;
   for (int it = 0;; ++it) {
     const int slot = it % nstg;
@@ -473,29 +491,29 @@ __global__ void __launch_bounds__(GGT, 1) gather_kernel(const SolveGroup* __rest
       const int rg = 2 * warp + (lane >> 4), cg = lane & 15;
 #pragma unroll 2
       for (int c = cg; c < b; c += 16) {
-        C v[RCMAX];
+        C v[RC];
 #pragma unroll
-        for (int j = 0; j < RCMAX; ++j) v[j] = V[j * ldv + c];
+        for (int j = 0; j < RC; ++j) v[j] = V[j * ldv + c];
 #pragma unroll
         for (int a = 0; a < NA; ++a) {
           const C m = M[(rg + 32 * a) * b + c];
 #pragma unroll
-          for (int j = 0; j < RCMAX; ++j) acc[a][j] = cfma(m, v[j], acc[a][j]);
+          for (int j = 0; j < RC; ++j) acc[a][j] = cfma(m, v[j], acc[a][j]);
         }
       }
     } else {
       const int rg8 = warp & 7, chalf = (warp >> 3) * (b / 2);
 #pragma unroll 2
       for (int r = 8 * rg8; r < 8 * rg8 + 8; ++r) {
-        C v[RCMAX];
+        C v[RC];
 #pragma unroll
-        for (int j = 0; j < RCMAX; ++j) v[j] = V[j * ldv + r];
+        for (int j = 0; j < RC; ++j) v[j] = V[j * ldv + r];
 #pragma unroll
         for (int a = 0; a < NA; ++a) {
           if (lane + 32 * a < b / 2) {
             const C m = M[r * b + chalf + lane + 32 * a];
 #pragma unroll
-            for (int j = 0; j < RCMAX; ++j) acc[a][j] = cfma(m, v[j], acc[a][j]);
+            for (int j = 0; j < RC; ++j) acc[a][j] = cfma(m, v[j], acc[a][j]);
           }
         }
       }
@@ -509,55 +527,43 @@ __global__ void __launch_bounds__(GGT, 1) gather_kernel(const SolveGroup* __rest
         ++inflight;
       }
       if (mt.end) {
-        // reduce-scatter over the 16 lanes of a row group: value q = a * 8 + j; after the stage
-        // with offset o a lane keeps the half selected by its bit o, so lane cg ends with q = cg
+        constexpr int NV = NA * RC, REP = 16 / NV;
         C* f = &acc[0][0];
-#pragma unroll
-        for (int o = 8, n = 16; o >= 1; o >>= 1, n >>= 1) {
-          const bool up = (lane & o) != 0;
-#pragma unroll
-          for (int q = 0; q < n / 2; ++q) {
-            const C lo = f[q], hi = f[q + n / 2];
-            const C send = up ? lo : hi;
-            C keep = up ? hi : lo;
-            keep = cadd(keep, shfl_xor_c(send, o));
-            f[q] = keep;
-          }
-        }
+        lane_scatter<NV>(f, lane);
         const int rg = 2 * warp + (lane >> 4), cg = lane & 15;
-        const int a = cg >> 3, j = cg & 7;
-        if (j < rc)
+        const int q = cg / REP, a = q / RC, j = q % RC;
+        if (j < rc && cg % REP == 0)
           P[(int64_t)mt.slot * nh * b * nrhs + (int64_t)(mt.h * HR + rg + 32 * a) * nrhs + j0 + j] = f[0];
 #pragma unroll
         for (int a2 = 0; a2 < NA; ++a2)
 #pragma unroll
-          for (int j2 = 0; j2 < RCMAX; ++j2) acc[a2][j2] = CT<R>::make(0, 0);
+          for (int j2 = 0; j2 < RC; ++j2) acc[a2][j2] = CT<R>::make(0, 0);
       }
     } else {
       if (mt.end) {
         // sum the 8 row groups of every (column, rhs) in a fixed order, in the consumed slot
-        C* red = sbase + (int64_t)slot * stg;            // [8][b][RCMAX], within the tile part
+        C* red = sbase + (int64_t)slot * stg;            // [8][b][RC], within the tile part
         const int rg8 = warp & 7, chalf = (warp >> 3) * (b / 2);
 #pragma unroll
         for (int a = 0; a < NA; ++a) {
           const int c = chalf + lane + 32 * a;
           if (lane + 32 * a < b / 2)
 #pragma unroll
-            for (int j = 0; j < RCMAX; ++j) red[(rg8 * b + c) * RCMAX + j] = acc[a][j];
+            for (int j = 0; j < RC; ++j) red[(rg8 * b + c) * RC + j] = acc[a][j];
         }
         __syncthreads();
         C* out = P + ((int64_t)mt.slot * nh + mt.h) * b * nrhs + j0;
-        for (int o = threadIdx.x; o < b * RCMAX; o += GGT) {
-          const int c = o / RCMAX, j = o % RCMAX;
-          C v = red[c * RCMAX + j];
+        for (int o = threadIdx.x; o < b * RC; o += GGT) {
+          const int c = o / RC, j = o % RC;
+          C v = red[c * RC + j];
 #pragma unroll
-          for (int w = 1; w < 8; ++w) v = cadd(v, red[(w * b + c) * RCMAX + j]);
+          for (int w = 1; w < 8; ++w) v = cadd(v, red[(w * b + c) * RC + j]);
           if (j < rc) out[(int64_t)c * nrhs + j] = v;
         }
 #pragma unroll
         for (int a = 0; a < NA; ++a)
 #pragma unroll
-          for (int j = 0; j < RCMAX; ++j) acc[a][j] = CT<R>::make(0, 0);
+          for (int j = 0; j < RC; ++j) acc[a][j] = CT<R>::make(0, 0);
         __syncthreads();                                 // the slot is free again
       }
       if (warp == 0 && pu < nunits) {
@@ -762,7 +768,7 @@ __global__ void __launch_bounds__(GT) block_fwd_kernel(BlockSweep s, const typen
       const int h = q % nh;
       if (q < nh) {
         // y_t rows [h*64, h*64+64) = Linv_t[rows] r_t
-        rows_matvec<R, 0>(cur, ldl, b, sv + (int64_t)t * b * ldv, ldv, rc, sy + h * HR * ldv, ldv);
+        rows_matvec<R, 0, RCMAX>(cur, ldl, b, sv + (int64_t)t * b * ldv, ldv, rc, sy + h * HR * ldv, ldv);
         if (q == nh - 1) {
           __syncthreads();
           for (int i = threadIdx.x; i < b * rc; i += GT) {
@@ -772,7 +778,7 @@ __global__ void __launch_bounds__(GT) block_fwd_kernel(BlockSweep s, const typen
         }
       } else {
         const int tp = t + 1 + (q - nh) / nh;
-        rows_matvec<R, 2>(cur, ldl, b, sy, ldv, rc, sv + (int64_t)(tp * b + h * HR) * ldv, ldv);
+        rows_matvec<R, 2, RCMAX>(cur, ldl, b, sy, ldv, rc, sv + (int64_t)(tp * b + h * HR) * ldv, ldv);
       }
       __syncthreads();
     }
@@ -847,7 +853,7 @@ __global__ void __launch_bounds__(GT) block_bwd_kernel(BlockSweep s, const typen
       const int h = q % nh;
       if (q < nh) {
         // w_t += Linv_t[rows of half h]^T r_t[rows of half h]
-        cols_matvec<R, 1>(cur, ldl, b, sv + (int64_t)(t * b + h * HR) * ldv, ldv, rc, sy, ldv);
+        cols_matvec<R, 1, RCMAX>(cur, ldl, b, sv + (int64_t)(t * b + h * HR) * ldv, ldv, rc, sy, ldv);
         if (q == nh - 1) {
           __syncthreads();
           for (int i = threadIdx.x; i < b * rc; i += GT) {
@@ -858,7 +864,7 @@ __global__ void __launch_bounds__(GT) block_bwd_kernel(BlockSweep s, const typen
       } else {
         // tile (t0+t, t0+tp): r_tp[c] -= sum_{r in half h} L[r][c] w_t[r]
         const int tp = (q - nh) / nh;
-        cols_matvec<R, 2>(cur, ldl, b, sy + h * HR * ldv, ldv, rc, sv + (int64_t)tp * b * ldv, ldv);
+        cols_matvec<R, 2, RCMAX>(cur, ldl, b, sy + h * HR * ldv, ldv, rc, sv + (int64_t)tp * b * ldv, ldv);
       }
       __syncthreads();
     }
@@ -918,30 +924,30 @@ __device__ __forceinline__ void stage_rows(C* dst, int ldd, const C* src, int ld
 
 // dst[c][j] (=, +=, or -= by MODE 0 / 1 / 2) sum_{r < nrows} M[r][c] V[r][j] for the 64 columns of
 // a staged column strip
-template <typename R, int MODE>
+template <typename R, int MODE, int RC>
 __device__ __forceinline__ void colstrip_matvec(const typename CT<R>::C* M, int ldm, int nrows,
                                                 const typename CT<R>::C* V, int ldv, int rc,
                                                 typename CT<R>::C* dst, int ldd) {
   using C = typename CT<R>::C;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = warp * 8 + (lane >> 2), rq = lane & 3;
-  C acc[RCMAX];
+  C acc[RC];
 #pragma unroll
-  for (int j = 0; j < RCMAX; ++j) acc[j] = CT<R>::make(0, 0);
+  for (int j = 0; j < RC; ++j) acc[j] = CT<R>::make(0, 0);
 #pragma unroll 4
   for (int r = rq; r < nrows; r += 4) {
     const C m = M[r * ldm + c];
     const C* v = V + r * ldv;
-    C vv[RCMAX];
+    C vv[RC];
 #pragma unroll
-    for (int j = 0; j < RCMAX; ++j) vv[j] = (j < rc) ? v[j] : CT<R>::make(0, 0);
+    for (int j = 0; j < RC; ++j) vv[j] = (j < rc) ? v[j] : CT<R>::make(0, 0);
 #pragma unroll
-    for (int j = 0; j < RCMAX; ++j) acc[j] = cfma(m, vv[j], acc[j]);
+    for (int j = 0; j < RC; ++j) acc[j] = cfma(m, vv[j], acc[j]);
   }
-  quad_reduce(acc);
+  quad_reduce<RC>(acc);
   if (rq == 0) {
 #pragma unroll
-    for (int j = 0; j < RCMAX; ++j)
+    for (int j = 0; j < RC; ++j)
       if (j < rc)
         dst[c * ldd + j] = MODE == 0 ? acc[j] : (MODE == 1 ? cadd(dst[c * ldd + j], acc[j]) : csub(dst[c * ldd + j], acc[j]));
   }
@@ -977,7 +983,7 @@ constexpr int EXT_REDUCE = 12;    // partials per row above which a level gets a
 //   y_J = L_JJ^{-1} r_J (forward),  w_J = L_JJ^{-T} r_J (backward),
 // so every CTA only needs the whole r_J (one exchange through distributed shared memory) and
 // its own strips of the inverse: no sequential steps and no barriers between them.
-template <typename R, bool FWD, bool INV>
+template <typename R, bool FWD, bool INV, int RC>
 __global__ void __launch_bounds__(GT) chain_kernel(ChainSweep s, const typename CT<R>::C* __restrict__ L,
                                                    const typename CT<R>::C* __restrict__ Linv,
                                                    typename CT<R>::C* __restrict__ Y) {
@@ -1151,8 +1157,8 @@ __global__ void __launch_bounds__(GT) chain_kernel(ChainSweep s, const typename 
         const C* M = next_stage();
         const C* V = sR + (int64_t)(FWD ? q : tq + q) * b * ldv;
         if (!bad) {
-          if (q == 0) rows_matvec_dense<R, 0>(M, b, V, ldv, rc, o, ldv);
-          else rows_matvec_dense<R, 1>(M, b, V, ldv, rc, o, ldv);
+          if (q == 0) rows_matvec_dense<R, 0, RC>(M, b, V, ldv, rc, o, ldv);
+          else rows_matvec_dense<R, 1, RC>(M, b, V, ldv, rc, o, ldv);
         }
         __syncthreads();
       }
@@ -1177,8 +1183,8 @@ __global__ void __launch_bounds__(GT) chain_kernel(ChainSweep s, const typename 
         const C* M = next_stage();
         C* o = obuf + (int64_t)l * HR * ldv;
         if (!bad) {
-          if (FWD) rows_matvec<R, 0>(M, ldst, b, sy, ldv, rc, o, ldv);
-          else colstrip_matvec<R, 0>(M, ldst, b, sy, ldv, rc, o, ldv);
+          if (FWD) rows_matvec<R, 0, RC>(M, ldst, b, sy, ldv, rc, o, ldv);
+          else colstrip_matvec<R, 0, RC>(M, ldst, b, sy, ldv, rc, o, ldv);
         }
         __syncthreads();
         for (int i = threadIdx.x; i < HR * rc; i += GT) {
@@ -1203,8 +1209,8 @@ __global__ void __launch_bounds__(GT) chain_kernel(ChainSweep s, const typename 
         const C* M = next_stage();
         C* r = rbuf + (int64_t)l * HR * ldv;
         if (!bad) {
-          if (FWD) rows_matvec<R, 2>(M, ldst, b, sy, ldv, rc, r, ldv);
-          else colstrip_matvec<R, 2>(M, ldst, b, sy, ldv, rc, r, ldv);
+          if (FWD) rows_matvec<R, 2, RC>(M, ldst, b, sy, ldv, rc, r, ldv);
+          else colstrip_matvec<R, 2, RC>(M, ldst, b, sy, ldv, rc, r, ldv);
         }
         __syncthreads();
       }
@@ -1357,6 +1363,15 @@ static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+// f(std::integral_constant<int, rc>) for rc in {1, 2, 4, 8}
+template <typename F>
+static void with_rc(int rc, F f) {
+  if (rc == 1) f(std::integral_constant<int, 1>{});
+  else if (rc == 2) f(std::integral_constant<int, 2>{});
+  else if (rc == 4) f(std::integral_constant<int, 4>{});
+  else f(std::integral_constant<int, 8>{});
+}
+
 template <typename R>
 static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
   using C = typename CT<R>::C;
@@ -1378,9 +1393,20 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
   const size_t gstage = sizeof(C) * ((size_t)HR * b + (size_t)RCMAX * (b + 16 / sizeof(C)));
   const int gstg = (int)std::max<size_t>(1, std::min<size_t>(GMAXSTG, SWEEP_SMEM_LIMIT / gstage));
   const size_t gsm = (size_t)gstg * gstage;
-  const unsigned gy = (unsigned)((a.nrhs + RCMAX - 1) / RCMAX);
-  cudaFuncSetAttribute(gather_kernel<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
-  cudaFuncSetAttribute(gather_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
+  // Right-hand sides per block: the products run over a compile-time count RC (a power of two), so that
+  // few right-hand sides do not pay for eight.  FP64 products are bound by the FP64 pipe (a 64 x 64 tile
+  // times 8 right-hand sides holds an SM for 43 us), so there the right-hand sides are also spread over
+  // more blocks while a level leaves SMs idle; FP32 ones are bound by the tile's loads, which that would
+  // repeat.  FP64 sweeps of a 4 x 4 grid, m = 512, 8 right-hand sides: 13.8 -> 7.7 ms; 3 x 3, m = 100, 3
+  // right-hand sides: 2.4 -> 0.54 ms; complex64, 8 x 8, m = 256, 1 right-hand side: 3.3 -> 2.8 ms.
+  int rmax = 1;
+  while (rmax < a.nrhs && rmax < RCMAX) rmax <<= 1;
+  const int64_t nsm_rc = sizeof(R) == 8 ? a.nsm : 0;
+  auto pick_rc = [&](int64_t blocks) {
+    int rc = rmax;
+    while (rc > 1 && blocks * ((a.nrhs + rc / 2 - 1) / (rc / 2)) <= nsm_rc) rc >>= 1;
+    return rc;
+  };
   int nsm = 0;
   {
     int dev = 0;
@@ -1396,17 +1422,18 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
       return;
     }
     const int nunits = (int)((i1 - i0) * nh);
-    const dim3 grid((unsigned)std::min<int64_t>(nunits, nsm), gy);
-    if (fwd)
-      launch_pdl(gather_kernel<R, true>, grid, dim3(GGT), gsm, st, a.fwd_groups + i0, a.fwd_items, L, Y, P, a.npad, b,
-                 a.nrhs, a.status, mk, nunits, gstg);
-    else
-      launch_pdl(gather_kernel<R, false>, grid, dim3(GGT), gsm, st, a.bwd_groups + i0, a.bwd_items, L, Y, P, a.npad, b,
-                 a.nrhs, a.status, mk, nunits, gstg);
+    const int rc = pick_rc(nunits);
+    with_rc(rc, [&](auto k) {
+      constexpr int RC = decltype(k)::value;
+      auto kern = fwd ? gather_kernel<R, true, RC> : gather_kernel<R, false, RC>;
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
+      launch_pdl(kern, dim3((unsigned)std::min<int64_t>(nunits, nsm), (unsigned)((a.nrhs + RC - 1) / RC)), dim3(GGT), gsm, st,
+                 (fwd ? a.fwd_groups : a.bwd_groups) + i0, fwd ? a.fwd_items : a.bwd_items, L, Y, P, a.npad, b, a.nrhs,
+                 a.status, mk, nunits, gstg);
+    });
   };
   // cluster chains: usable when every level's largest block fits CHAIN_MAXCL x CHAIN_MAXLOC strips
-  const int crc = a.nrhs < RCMAX ? a.nrhs : RCMAX;
-  const int cldv = vec_ld(crc);
+  const int cldv = vec_ld(rmax);
   const int cstg = std::max(HR * stage_ld<C>(b), b * stage_ld<C>(HR));
   bool chain = a.lev_maxnt != nullptr;
   int max_loc = 1;
@@ -1427,13 +1454,6 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
   if (chain && chain_smem(max_loc) > SWEEP_SMEM_LIMIT) chain = false;
   if (inv && !chain) return (int)cudaErrorInvalidConfiguration;   // the host enables INV only where it fits
   if (chain) {
-    if (inv) {
-      cudaFuncSetAttribute(chain_kernel<R, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(max_loc));
-      cudaFuncSetAttribute(chain_kernel<R, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(max_loc));
-    } else {
-      cudaFuncSetAttribute(chain_kernel<R, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(max_loc));
-      cudaFuncSetAttribute(chain_kernel<R, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(max_loc));
-    }
     ChainSweep cs;
     cs.status = a.status;
     cs.tstart = a.tstart;
@@ -1456,8 +1476,9 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
       cs.nloc = (S + cs.cl - 1) / cs.cl;
       cs.blocks = a.lev_blocks + a.lev_ptr[lv];
       const unsigned nb = (unsigned)(a.lev_ptr[lv + 1] - a.lev_ptr[lv]);
-      cs.rc = crc;
-      const unsigned ny = (unsigned)((a.nrhs + crc - 1) / crc);
+      const int rc = pick_rc((int64_t)nb * cs.cl);
+      cs.rc = rc < a.nrhs ? rc : a.nrhs;
+      const unsigned ny = (unsigned)((a.nrhs + cs.rc - 1) / cs.rc);
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(nb * (unsigned)cs.cl, ny, 1);
       cfg.blockDim = dim3(GT, 1, 1);
@@ -1473,11 +1494,16 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
       cfg.attrs = attr;
       cfg.numAttrs = 2;
       ++a.launches;
-      if (inv)
-        return fwd ? cudaLaunchKernelEx(&cfg, chain_kernel<R, true, true>, cs, L, Linv, Y)
-                   : cudaLaunchKernelEx(&cfg, chain_kernel<R, false, true>, cs, L, Linv, Y);
-      return fwd ? cudaLaunchKernelEx(&cfg, chain_kernel<R, true, false>, cs, L, Linv, Y)
-                 : cudaLaunchKernelEx(&cfg, chain_kernel<R, false, false>, cs, L, Linv, Y);
+      cudaError_t e = cudaSuccess;
+      with_rc(rc, [&](auto k) {
+        constexpr int RC = decltype(k)::value;
+        auto kern = fwd ? chain_kernel<R, true, false, RC> : chain_kernel<R, false, false, RC>;
+        if constexpr (sizeof(R) == 4)          // the host builds inverses for complex64 factors only
+          if (inv) kern = fwd ? chain_kernel<R, true, true, RC> : chain_kernel<R, false, true, RC>;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(max_loc));
+        e = cudaLaunchKernelEx(&cfg, kern, cs, L, Linv, Y);
+      });
+      return e;
     };
     for (int lv = 0; lv < a.nlevels; ++lv) {
       const int64_t i0 = a.fwd_group_ptr[lv], i1 = a.fwd_group_ptr[lv + 1];
