@@ -64,7 +64,7 @@ enum {
 enum {
   D3M_FP64 = 0,          /* complex128 factors, no refinement; tile products as exact digit products
                             on tcgen05 tensor cores accumulated in fixed point and rounded once to FP64
-                            (with pivoting, or where the device memory is short: an FP64 SIMT engine) */
+                            (where the device memory is short of them, or a task lists over 64 products: an FP64 SIMT engine) */
   D3M_MIXED_BF16X3 = 1,  /* complex64 factors; Schur/TRSM products on tcgen05 tensor cores as
                             split-BF16x3 (a = a_hi + a_lo; hi*hi + hi*lo + lo*hi) with FP32
                             accumulation in TMEM; FP64 residual + iterative refinement */
@@ -119,8 +119,8 @@ typedef struct {
   int32_t pivot;            /* 1 = Bunch-Kaufman symmetric pivoting (1 x 1 and 2 x 2 pivots, the
                                paper's sytrf, Sec. II) inside every diagonal tile: the tile is
                                factored as S = Lt D Lt^T, Lt = P^T L; the block structure and task
-                               graph are unchanged.  SIMT engines only (D3M_FP64, which then runs
-                               its SIMT engine, and D3M_MIXED_SIMT32; D3M_ERR_INVALID otherwise).  0 (default) =
+                               graph are unchanged.  D3M_FP64 and D3M_MIXED_SIMT32 only
+                               (D3M_ERR_INVALID otherwise).  0 (default) =
                                unpivoted, scalar D */
 } d3m_options;
 

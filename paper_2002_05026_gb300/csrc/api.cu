@@ -21,7 +21,7 @@ struct d3m_ctx {
   Symbolic S;
   d3m_options opt{};
   bool fp64 = true, tc = false, tf32 = false;
-  bool dig = false;                  // FP64 unpivoted: tile products as exact digit products (factor_dig.cu)
+  bool dig = false;                  // FP64: tile products as exact digit products (factor_dig.cu)
   bool resid = true;                 // the residual's buffers and digit planes exist
   int b = 64;
   int device = 0, nsm = 0;
@@ -785,10 +785,10 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
   CUDA_TRY(h, cudaMemset(h->sweep_status, 0, sizeof(int)));
   ALLOC(h->contract, double2, S.N);
   CUDA_TRY(h, cudaMallocHost(&h->h_stat, 3 * sizeof(double)));
-  // FP64 without pivoting: the digit engine, where its words (16 bytes per complex entry of L and of
+  // FP64: the digit engine, where its words (16 bytes per complex entry of L and of
   // W, beside L itself) leave a quarter of the free memory to the caller; else the SIMT engine,
   // which needs none of them
-  if (h->fp64 && !h->opt.pivot) {
+  if (h->fp64) {
     const size_t words = (size_t)ntiles * 2 * b * b * sizeof(unsigned long long), exps = (size_t)ntiles * b;
     size_t mfree = 0, mtotal = 0;
     if (cudaMemGetInfo(&mfree, &mtotal) != cudaSuccess) cudaGetLastError();

@@ -1,5 +1,5 @@
 // Persistent block-DAG factorization in FP64 with the tile products on the tensor cores (tile
-// edge 64, complex128 factors, unpivoted): the D3M_FP64 engine.
+// edge 64, complex128 factors): the D3M_FP64 engine.
 //
 // GB300 issues two FP64 FMAs per clock and SM, so one 64 x 64 x 64 complex tile product is 1.05 M
 // DFMA = 0.25 ms of an SM, and both a task graph's throughput and its critical path are bound by
@@ -42,6 +42,7 @@
 #include <cuda_runtime.h>
 
 #include "device.cuh"
+#include "diag_bk.cuh"
 #include "kernels.h"
 
 namespace d3m {
@@ -154,6 +155,12 @@ __device__ __forceinline__ unsigned long long word_of(double x, int shift, int E
 // multiplies L[r][k] by s_r / s_k, leaves every row of an operand with one scale
 __device__ __forceinline__ int balance_of(double2 d) {
   const int m = max(exp_of(d.x, 0), exp_of(d.y, 0));
+  return (m <= X_ZERO || m >= X_BAD) ? 0 : (m - 1023) >> 1;
+}
+// the same for a column of a 2 x 2 pivot block (or three times the same pivot)
+__device__ __forceinline__ int pair_balance(double2 d1, double2 d2, double2 e) {
+  const int m = max(max(max(exp_of(d1.x, 0), exp_of(d1.y, 0)), max(exp_of(d2.x, 0), exp_of(d2.y, 0))),
+                    max(exp_of(e.x, 0), exp_of(e.y, 0)));
   return (m <= X_ZERO || m >= X_BAD) ? 0 : (m - 1023) >> 1;
 }
 // digits of byte `sel` of two words (lo or hi halves x, y) as packed bf16: 128 + low 7 bits minus
@@ -336,6 +343,9 @@ using I64 = IntC<64>;
 
 }  // namespace
 
+// PIV: Bunch-Kaufman pivoting inside the diagonal tiles (diag_bk.cuh): Lt = P^T L, X = Lt^{-1} with its
+// columns in the tile's own order, D with 2 x 2 blocks; the products are the same
+template <bool PIV>
 __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams p) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (su(smem_raw) & 1023u)) & 1023u);
@@ -347,7 +357,8 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
   __shared__ const int32_t *s_ea[MAXP], *s_eb[MAXP];
   __shared__ short s_ex[MAXP][2 * TB];            // row scales of every product of the task
   __shared__ int s_eL[TB], s_eW[TB];              // scales (biased exponents first) of finished rows
-  __shared__ int s_ek[TB];                        // balance of every column
+  __shared__ int s_ek[TB], s_eS[TB];              // balance of every column; the same in the tile's order
+  __shared__ BkShared<double2> s_bk;              // pivot mode
   __shared__ double2 s_d[TB], s_dinv[TB], s_u[2][PW], s_x[2][PW], s_dg[2];
   __shared__ double2 sX[PW][PW + 1];              // inverse of a panel's diagonal block
   __shared__ float s_red[NWK];
@@ -602,6 +613,9 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if (lane == 0) s_red[warp] = mx;
       }
+      if constexpr (PIV) {
+        bk_factor<double, NTHR>(sS, LDS, s_bk);
+      } else {
       // one digit product of operands in shared memory (16 columns, nrow rows of the L side):
       // value(w_side, row, q, part) 2^(-+ balance of column q) (W side -, L side +)
       auto local_product = [&](auto nrow, int c0, auto value) {
@@ -775,12 +789,23 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         }
         __syncthreads();
       }
+      }
       if (__syncthreads_or(failed)) {
         if (tid == 0) set_error(p.ctl, D3M_ERR_TIMEOUT, task);
         break;
       }
-      // rows of padding are rows of the identity
-      if (tid < TB && tid >= nr) {
+      if constexpr (PIV) {
+        if (tid < TB) {
+          s_d[tid] = s_bk.d[tid];
+          // a 2 x 2 block's two columns share the balance of its largest entry
+          double2 m = s_bk.d[tid];
+          const bool first2 = s_bk.e[tid].x != 0 || s_bk.e[tid].y != 0;
+          const bool second2 = tid > 0 && (s_bk.e[tid - 1].x != 0 || s_bk.e[tid - 1].y != 0);
+          s_ek[tid] = pair_balance(m, first2 ? s_bk.d[tid + 1] : (second2 ? s_bk.d[tid - 1] : m),
+                                   first2 ? s_bk.e[tid] : (second2 ? s_bk.e[tid - 1] : m));
+        }
+      } else if (tid < TB && tid >= nr) {
+        // rows of padding are rows of the identity
         s_d[tid] = make_double2(1.0, 0.0);
         s_ek[tid] = 0;
       }
@@ -797,7 +822,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             const int s = lane + 32 * q;
-            x[q] = (s < r && r < nr) ? sS[s * LDS + r] : make_double2(s == r ? 1.0 : 0.0, 0.0);
+            x[q] = (s < r && (PIV || r < nr)) ? sS[s * LDS + r] : make_double2(s == r ? 1.0 : 0.0, 0.0);
             m = max(m, max(exp_of(x[q].x, s_ek[s]), exp_of(x[q].y, s_ek[s])));
           }
           m = __reduce_max_sync(0xffffffffu, m);
@@ -805,31 +830,41 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
           if (lane == 0) EL[(int64_t)T.tile * TB + r] = E;
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
-            const int s = lane + 32 * q;
-            Li[r * TB + s] = x[q];
-            f[word_at(r, s, 0)] = word_of(x[q].x, s_ek[s], E);
-            f[word_at(r, s, 1)] = word_of(x[q].y, s_ek[s], E);
+            const int s = lane + 32 * q, k = PIV ? s_bk.perm[s] : s;   // column k of X = Lt^{-1}
+            Li[r * TB + k] = x[q];
+            f[word_at(r, k, 0)] = word_of(x[q].x, s_ek[s], E);
+            f[word_at(r, k, 1)] = word_of(x[q].y, s_ek[s], E);
           }
         }
         double2* Lt = Lg + (int64_t)T.tile * TB * TB;
         for (int i = tid; i < TB * TB; i += NTHR) {
           const int r = i >> 6, c = i & 63;
-          Lt[i] = (c < r && r < nr) ? sS[r * LDS + c] : make_double2(c == r ? 1.0 : 0.0, 0.0);
+          Lt[(PIV ? s_bk.perm[r] : r) * TB + c] = (c < r && (PIV || r < nr)) ? sS[r * LDS + c] : make_double2(c == r ? 1.0 : 0.0, 0.0);
         }
-        if (tid < TB) Dg[(int64_t)T.col * TB + tid] = s_d[tid];
+        if (tid < TB) {
+          Dg[(int64_t)T.col * TB + tid] = s_d[tid];
+          if (PIV) {
+            reinterpret_cast<double2*>(p.E)[(int64_t)T.col * TB + tid] = s_bk.e[tid];
+            p.piv[(int64_t)T.col * TB + tid] = s_bk.perm[tid];
+          }
+        }
         if (warp == 0) {
           float smx = 0.f;
           for (int w = 0; w < NWK; ++w) smx = fmaxf(smx, s_red[w]);
           const double smax = scale2((double)sqrtf(smx), mexp - 1023);
           double amin = 3.0e38, amax = 0.0;
-          for (int c = lane; c < T.cv; c += 32) {
-            const double a = sqrt(cabs2(s_d[c]));
-            amin = fmin(amin, a);
-            amax = fmax(amax, a);
-          }
-          for (int o = 16; o > 0; o >>= 1) {
-            amin = fmin(amin, __shfl_xor_sync(0xffffffffu, amin, o));
-            amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+          if constexpr (PIV) {
+            bk_pivot_range<double>(s_bk, T.cv, amin, amax);
+          } else {
+            for (int c = lane; c < T.cv; c += 32) {
+              const double a = sqrt(cabs2(s_d[c]));
+              amin = fmin(amin, a);
+              amax = fmax(amax, a);
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+              amin = fmin(amin, __shfl_xor_sync(0xffffffffu, amin, o));
+              amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+            }
           }
           if (lane == 0) {
             record_pivot_stats(p.ctl, (float)amin, (float)amax);
@@ -846,12 +881,30 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         s_eW[tid] = X_ZERO;
         const double2 d = ld_cg(Dg + (int64_t)T.col * TB + tid);
         s_d[tid] = d;
-        s_ek[tid] = balance_of(d);
-        s_rec[tid] = 1.0 / (d.x * d.x + d.y * d.y);
+        if constexpr (PIV) {
+          // D^{-1}: [w_c w_(c+1)] [[d1, e], [e, d2]]^{-1}; s_u2 = the weight of the other column of a block
+          const double2* Eg = reinterpret_cast<const double2*>(p.E) + (int64_t)T.col * TB;
+          const double2 zero = make_double2(0.0, 0.0);
+          const double2 e0 = ld_cg(Eg + tid), e1 = tid > 0 ? ld_cg(Eg + tid - 1) : zero;
+          const bool first2 = e0.x != 0 || e0.y != 0, second2 = e1.x != 0 || e1.y != 0;
+          const double2 o = first2 || second2 ? ld_cg(Dg + (int64_t)T.col * TB + (first2 ? tid + 1 : tid - 1)) : d;
+          const double2 e = first2 ? e0 : (second2 ? e1 : zero);
+          const double2 det = first2 || second2 ? csub(cmul(d, o), cmul(e, e)) : d;
+          s_bk.u1[tid] = first2 || second2 ? cdiv(o, det) : cdiv(make_double2(1.0, 0.0), d);
+          s_bk.u2[tid] = first2 || second2 ? cdiv(make_double2(-e.x, -e.y), det) : zero;
+          s_bk.perm[tid] = first2 ? tid + 1 : (second2 ? tid - 1 : tid);
+          const int bal = pair_balance(d, o, first2 || second2 ? e : d);
+          s_ek[tid] = bal;
+          // the contraction of the triangular solve runs over the tile's own order
+          s_eS[p.piv[(int64_t)T.col * TB + tid]] = bal;
+        } else {
+          s_ek[tid] = s_eS[tid] = balance_of(d);
+          s_rec[tid] = 1.0 / (d.x * d.x + d.y * d.y);
+        }
       }
       __syncthreads();
       {
-        const int bal = s_ek[oc];
+        const int bal = s_eS[oc];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           const int m = __reduce_max_sync(0xffffffffu, exp_of(S[i], -bal));
@@ -894,7 +947,12 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         for (int i = 0; i < 8; ++i) {
           const int r = wr + 8 * i;
           w[i] = make_double2(sW[r * LDS + c], sW[(TB + r) * LDS + c]);
-          l[i] = make_double2((w[i].x * d.x + w[i].y * d.y) * rec, (w[i].y * d.x - w[i].x * d.y) * rec);
+          if constexpr (PIV) {
+            const int o = s_bk.perm[c];
+            l[i] = cfma(make_double2(sW[r * LDS + o], sW[(TB + r) * LDS + o]), s_bk.u2[c], cmul(w[i], s_bk.u1[c]));
+          } else {
+            l[i] = make_double2((w[i].x * d.x + w[i].y * d.y) * rec, (w[i].y * d.x - w[i].x * d.y) * rec);
+          }
           Lt[r * TB + c] = l[i];
           const int bw = __reduce_max_sync(0xffffffffu, max(exp_of(w[i].x, -bal), exp_of(w[i].y, -bal)));
           const int bl = __reduce_max_sync(0xffffffffu, max(exp_of(l[i].x, bal), exp_of(l[i].y, bal)));
@@ -938,9 +996,10 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
 
 int launch_factor_dig(const FactorParams& p, int nblocks, cudaStream_t st) {
   const size_t smem = SMEM_BYTES + 1024;   // + alignment slack
-  const cudaError_t e = cudaFuncSetAttribute(factor_dig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto kern = p.pivot ? factor_dig_kernel<true> : factor_dig_kernel<false>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
-  factor_dig_kernel<<<nblocks, NTHR, smem, st>>>(p);
+  kern<<<nblocks, NTHR, smem, st>>>(p);
   return (int)cudaGetLastError();
 }
 
