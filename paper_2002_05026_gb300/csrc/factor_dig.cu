@@ -33,10 +33,10 @@
 // does not (8 levels x 64 columns fill the tensor memory).
 //
 // Measured on GB300, factorization of a 4 x 4 grid with m = 512 (127 k products): 255 ms with DFMA tile
-// products (1.04 TFLOP/s, 83 % of the FP64 pipe), 22 ms here; 3 x 3 grid with m = 100: 12.3 -> 3.0 ms.  A
-// product takes 22 k cycles (DFMA: 524 k): 15 k for the four stages (MMAs and the expansion's 84 KB of
-// shared-memory stores share its bandwidth), 7 k for the read-back.  A diagonal tile takes about 130 us,
-// 16 us of it per 16-column pivot chain.  Solutions against 64-bit references: as far off as with DFMA
+// products (1.04 TFLOP/s, 83 % of the FP64 pipe), 20 ms here; 3 x 3 grid with m = 100: 12.3 -> 2.9 ms.  A
+// product takes about 20 k cycles (DFMA: 524 k), 8.7 k of them MMAs: two stages do not hide the
+// expansion (2 k a stage) behind them, and the read-back (6 k) waits for the last one.  A diagonal tile
+// takes about 120 us, 16 us of it per 16-column pivot chain.  Solutions against 64-bit references: as far off as with DFMA
 // (1.4e-15 and 1.1e-15 for these two).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -485,9 +485,9 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         w = load_words((iW ? s_fb : s_fa)[c / NCH] + ((c % NCH) * 256 + item) * 8);
       };
       fetch_words(0);
-      // two stages of a product are expanded before the read-back of the product before it, which
-      // frees the tensor memory for their MMAs
-      for (int c = 0; c <= nst + 1 && !failed; ++c) {
+      // the first stage of a product is expanded before the read-back of the product before it, which
+      // frees the tensor memory for its MMAs; the second one while those run
+      for (int c = 0; c <= nst && !failed; ++c) {
         if (c < nst) {
           const uint32_t s = (it0 + c) % NSTG, use = (it0 + c) / NSTG;
           failed = !__all_sync(0xffffffffu, bar_wait(su(&bar_empty[s]), (use & 1) ^ 1, deadline));
@@ -497,14 +497,14 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
           if (lane == 0) bar_arrive(su(&bar_full[s]));
-          if (warp == ISSUER && (c < NCH || c % NCH >= 2)) {
+          if (warp == ISSUER && (c < NCH || c % NCH != 0)) {
             if (lane == 0) issue(c);
             failed = __any_sync(0xffffffffu, failed);
           }
         }
-        if (c >= NCH + 1 && (c - NCH - 1) % NCH == 0) {
+        if (c >= NCH && c % NCH == 0) {
           // ---- read back the levels of product e
-          const int e = (c - NCH - 1) / NCH;
+          const int e = c / NCH - 1;
           const int db = s_MB[oc] - s_ex[e][TB + oc];
           failed = !__all_sync(0xffffffffu, bar_wait(su(&bar_accf), tile_no & 1, deadline));
           if (failed) break;
@@ -515,10 +515,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
           if (lane == 0) bar_arrive(su(&bar_acce));
           ++tile_no;
           if (warp == ISSUER && (e + 1) * NCH < nst) {
-            if (lane == 0) {
-              issue((e + 1) * NCH);
-              if (!failed) issue((e + 1) * NCH + 1);
-            }
+            if (lane == 0) issue((e + 1) * NCH);
             failed = __any_sync(0xffffffffu, failed);
           }
         }
@@ -775,18 +772,27 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
           return -reinterpret_cast<const double*>(&sX[q][row - c0])[part];
         });
         if (failed) break;
-        if (r0 >= c1) read_levels(I16{}, I64{}, r0, [](int) { return 0; });
-        product_read();
-        if (r0 >= c1) {
+        // rows c1 .. 63 in groups of 4, a quarter of them to each of the four warps of an SM partition
+        {
+          const int per = (TB - c1) >> 2, rw = c1 + (warp >> 2) * per;
+#pragma unroll 1
+          for (int rb = rw; rb < rw + per; rb += 4) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int r = r0 + i;
-            if (oc <= r) {
-              double* t = reinterpret_cast<double*>(oc >= c1 ? sS + r * LDS + oc : sS + oc * LDS + r) + ri;
-              *t -= result(i);
+            for (int i = 0; i < 4; ++i) H[i] = Lo[i] = 0;
+            read_levels(I4{}, I64{}, rb, [](int) { return 0; });
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int r = rb + i;
+              if (oc <= r) {
+                const double v = max(s_MA[r], s_MB[oc]) >= E_BAD ? __longlong_as_double(0x7ff8000000000000ll)
+                                                                   : fixed_to_double(H[i], Lo[i], s_MA[r] + s_MB[oc] - 74);
+                double* t = reinterpret_cast<double*>(oc >= c1 ? sS + r * LDS + oc : sS + oc * LDS + r) + ri;
+                *t -= v;
+              }
             }
           }
         }
+        product_read();
         __syncthreads();
       }
       }
