@@ -29,6 +29,12 @@
 // (and claims the block's next ready task while they run), all 8 warps run the epilogues (warp w
 // reads TMEM lanes 32*(w%4).., columns half w/4), warp 2 releases a finished task's successors.
 // Diagonal tiles are factored (unpivoted LDL^T) and inverted with SIMT FP32 in shared memory.
+//
+// Small and medium systems are bound by the chain of diagonal and triangular-solve tasks, whose code runs
+// once per task and at the rate it is fetched (the kernel was 190 KB of instructions): the three kinds of
+// task share one loop that forms S and the K entries take one address each (142 KB), and a diagonal tile
+// skips its panels of padding.  Diagonal task 92 -> 69 us (m = 512), 82 -> 39 us (m = 64); factorizations: 3 x 3 x 3
+// grid of uneven blocks 5.7 -> 4.3 ms, 4 x 4 m = 512 4.3 -> 3.6, 8 x 8 m = 256 5.3 -> 4.4, 8 x 8 m = 512 13.4 -> 12.5.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -74,6 +80,7 @@ static_assert(Eng<true>::NSTAGE * stage_slot<true>() <= SMEM_BYTES && SMEM_T + 2
 static_assert((TB / Eng<false>::KC) * stage_a<false>() == SMEM_T && (TB / Eng<true>::KC) * stage_a<true>() == SMEM_T, "S");
 constexpr int LDS = 129;                        // c64 diagonal tile row stride (elements)
 constexpr uint32_t DIAG_AUX = 130 * 1024;       // d / column / scratch vectors of a diagonal task
+static_assert(DIAG_AUX + 8 * (TB + 32 * 97 + 2 * 32 * 33 + 2 * 32) <= SMEM_BYTES, "shared memory of a diagonal task");
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t ACC1 = 0, ACC2 = 256;        // TMEM columns of the two accumulators
 
@@ -271,8 +278,26 @@ __device__ __forceinline__ void load_s_in(const TileTask& T, const double2* K, f
       kin[2 * i + 1] = make_float2(v[i].z, v[i].w);
     }
   } else {
+    // K_IJ (padding: unit diagonal inside diagonal blocks; fill blocks: zero)
+    const int rr = T.r0 + r;
+    const bool row = T.k_off >= 0 && r < T.rv;
+    const int64_t stride = T.k_tr ? 1 : T.k_ld;
+    const double2* src = K + (row ? T.k_off + (T.k_tr ? (int64_t)rr * T.k_ld + T.c0 : (int64_t)T.c0 * T.k_ld + rr) + c0 * stride : 0);
+    const int nc = row ? T.cv - c0 : 0;             // entries of this row and range in the block
+    double2 v[32];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) kin[i] = k_entry<float>(T, K, r, c0 + i);
+    for (int i = 0; i < 32; ++i) {
+      v[i] = i < nc ? __ldg(src) : make_double2(0.0, 0.0);
+      src += stride;
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i) kin[i] = CT<float>::from(v[i]);
+    if ((T.flags & TF_SAME_BLOCK) && (T.rv < TB || T.cv < TB)) {
+      const int dg = rr - T.c0 - c0;                // position of the block's diagonal
+#pragma unroll
+      for (int i = 0; i < 32; ++i)
+        if (i == dg && i >= nc) kin[i].x = 1.f;
+    }
   }
 }
 
@@ -291,7 +316,8 @@ __device__ __forceinline__ void load_s_in(const TileTask& T, const double2* K, f
 // ends up, in the upper triangle, which starts at zero.  The diagonal block of panel k + 1 is
 // updated first, so that two warps factor it while the other six finish panel k's updates.
 constexpr int DW = 32;          // panel width
-constexpr int WT_LD = 96;       // row length of the W panel scratch (c-major: Wt[c][row - c1])
+constexpr int WT_LD = 97;       // row length of the W panel scratch (c-major: Wt[c][row - c1]; odd: the columns of a
+                                // warp's stores fall in distinct banks)
 constexpr int XD_LD = DW + 1;   // row length of the dense copies of X_kk (two, by panel parity)
 
 // The DW x DW diagonal block at (c0, c0), two warps: warp 0 factors it (lane i = row i), warp 1
@@ -309,12 +335,17 @@ __device__ __forceinline__ void ldlt_phase(float2 (&a)[DW], int j0, float2* sS, 
     // column goes through a shared buffer (one broadcast load per entry), two buffers by step parity.
     const float2 cj = a[0];
     float2* cb = colb + (j & 1) * DW;
-    cb[lane] = cj;
+    cb[(lane - j) & 31] = cj;                                // rotated: entry m is a_(j+m)[j]
     __syncwarp();
-    const float2 dj = cb[j];
+    const float4* c4 = reinterpret_cast<const float4*>(cb);
+    float4 c = c4[0];
+    const float2 dj = make_float2(c.x, c.y);
     const float2 l = cdiv(cj, dj);
 #pragma unroll
-    for (int m = 1; m < NM; ++m) a[m - 1] = cfms(l, cb[(j + m) & 31], a[m]);
+    for (int m = 1; m < NM; ++m) {
+      if (m % 2 == 0) c = c4[m / 2];
+      a[m - 1] = cfms(l, m % 2 ? make_float2(c.z, c.w) : make_float2(c.x, c.y), a[m]);
+    }
     a[NM - 1] = make_float2(0.f, 0.f);
     if (lane > j) sS[(c0 + lane) * LDS + c0 + j] = l;
     if (lane == j) s_d[c0 + j] = dj;
@@ -329,11 +360,9 @@ __device__ __forceinline__ void linv_phase(float2 (&x)[DW], int q0, float2* sS, 
     const float2 xq = x[0];
     if (q > lane) sS[(c0 + lane) * LDS + c0 + q] = xq;      // X[q][lane] at sS[c0 + lane][c0 + q]
     Xd[q * XD_LD + lane] = xq;                               // dense copy, zeros and ones included
-#pragma unroll
-    for (int m = 1; m < NM; ++m) {
-      const int row = min(q + m, DW - 1);                    // rows past the block feed unused slots
-      x[m - 1] = cfms(sS[(c0 + row) * LDS + c0 + q], xq, x[m]);
-    }
+    const float2* lq = sS + (c0 + q) * LDS + c0 + q;         // rows past the block (still shared memory of
+#pragma unroll                                               // the task) feed unused slots
+    for (int m = 1; m < NM; ++m) x[m - 1] = cfms(lq[m * LDS], xq, x[m]);
     x[NM - 1] = make_float2(0.f, 0.f);
   }
 }
@@ -367,71 +396,52 @@ __device__ __forceinline__ void diag_block_2warps(float2* sS, float2* s_d, float
 }
 
 
-// All threads: W_rk, L_rk for the rows below panel k (k < 3) and X_kj = -X_kk Z_kj (j < k).
+// All threads: V = sS[:, panel k] X_kk^T for the rows of the other panels (of np), one product for both kinds:
+// below the panel it is W_rk = A_rk X_kk^T (then L_rk = W_rk D_k^{-1}); above it, where the rows
+// hold the transposed Z_kj, it is -X_kj^T.
 __device__ __forceinline__ void diag_panel_solve(float2* sS, const float2* s_d, float2* Wt, const float2* Xd, int k,
-                                                 int tid) {
-  const int c0 = DW * k, c1 = c0 + DW, nrb = 3 - k;
-  // W: thread -> columns cg + 8 jj, rows c1 + rg + 32 ii
+                                                 int np, int tid) {
+  const int c0 = DW * k, c1 = c0 + DW;
+  // thread -> columns cg + 8 jj, rows rg + 32 i of the i-th other panel
   const int cg = tid & 7, rg = tid >> 3;
+  const float2* A[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) A[i] = sS + (rg + DW * min(i < k ? i : i + 1, np - 1)) * LDS + c0;
   float2 w[3][4];
 #pragma unroll
-  for (int ii = 0; ii < 3; ++ii)
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) w[ii][jj] = make_float2(0.f, 0.f);
-  if (nrb > 0) {
+    for (int jj = 0; jj < 4; ++jj) w[i][jj] = make_float2(0.f, 0.f);
 #pragma unroll 4
-    for (int q = 0; q < DW; ++q) {
-      float2 xq[4], aq[3];
+  for (int q = 0; q < DW; ++q) {
+    float2 xq[4], aq[3];
 #pragma unroll
-      for (int jj = 0; jj < 4; ++jj) xq[jj] = Xd[(cg + 8 * jj) * XD_LD + q];
+    for (int jj = 0; jj < 4; ++jj) xq[jj] = Xd[(cg + 8 * jj) * XD_LD + q];
 #pragma unroll
-      for (int ii = 0; ii < 3; ++ii) aq[ii] = ii < nrb ? sS[(c1 + rg + 32 * ii) * LDS + c0 + q] : make_float2(0.f, 0.f);
+    for (int i = 0; i < 3; ++i) aq[i] = A[i][q];
 #pragma unroll
-      for (int ii = 0; ii < 3; ++ii)
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) w[ii][jj] = cfma(aq[ii], xq[jj], w[ii][jj]);
-    }
-  }
-  // X_kj: thread -> rows a = (tid >> 5) + 8 i, column b = tid & 31
-  const int b = tid & 31, ar = tid >> 5;
-  float2 xo[3][4];
-#pragma unroll
-  for (int j = 0; j < 3; ++j)
-#pragma unroll
-    for (int i = 0; i < 4; ++i) xo[j][i] = make_float2(0.f, 0.f);
-  if (k > 0) {
-#pragma unroll 4
-    for (int q = 0; q < DW; ++q) {
-      float2 xa[4], z[3];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) xa[i] = Xd[(ar + 8 * i) * XD_LD + q];
-#pragma unroll
-      for (int j = 0; j < 3; ++j) z[j] = j < k ? sS[(DW * j + b) * LDS + c0 + q] : make_float2(0.f, 0.f);
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) xo[j][i] = cfma(xa[i], z[j], xo[j][i]);
-    }
+      for (int jj = 0; jj < 4; ++jj) w[i][jj] = cfma(aq[i], xq[jj], w[i][jj]);
   }
   __syncthreads();   // every A_rk and Z_kj has been read
-  if (nrb > 0) {
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      const int c = cg + 8 * jj;
-      const float2 dinv = cdiv(make_float2(1.f, 0.f), s_d[c0 + c]);
+  for (int jj = 0; jj < 4; ++jj) {
+    const int c = cg + 8 * jj;
+    const float2 dinv = cdiv(make_float2(1.f, 0.f), s_d[c0 + c]);
 #pragma unroll
-      for (int ii = 0; ii < 3; ++ii)
-        if (ii < nrb) {
-          sS[(c1 + rg + 32 * ii) * LDS + c0 + c] = cmul(w[ii][jj], dinv);
-          Wt[c * WT_LD + rg + 32 * ii] = w[ii][jj];
-        }
+    for (int i = 0; i < 3; ++i) {
+      if (i >= np - 1) continue;
+      const int r = rg + DW * (i < k ? i : i + 1);
+      float2* o = sS + r * LDS + c0 + c;
+      if (i < k) {
+        *o = make_float2(-w[i][jj].x, -w[i][jj].y);
+      } else {
+        *o = cmul(w[i][jj], dinv);
+        Wt[c * WT_LD + r - c1] = w[i][jj];
+      }
     }
   }
-#pragma unroll
-  for (int j = 0; j < 3; ++j)
-    if (j < k)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) sS[(DW * j + b) * LDS + c0 + ar + 8 * i] = make_float2(-xo[j][i].x, -xo[j][i].y);
   __syncthreads();
 }
 
@@ -461,9 +471,9 @@ __device__ __forceinline__ void diag_next_block(float2* sS, const float2* Wt, in
 // Warps 2..7 (t = thread index among them): the rest of panel k's updates as 32 x 32 block jobs --
 // trailing blocks (r, s), k < s <= r, other than (k+1, k+1), then Z blocks (r, j), r > k, j <= k.
 // A job is two chunks of 32 threads; each thread owns rows aa + 8 i and columns bb + 8 q (i, q < 4).
-__device__ __forceinline__ void diag_panel_update(float2* sS, const float2* Wt, const float2* Xd, int k, int t) {
+__device__ __forceinline__ void diag_panel_update(float2* sS, const float2* Wt, const float2* Xd, int k, int np, int t) {
   const int c0 = DW * k, c1 = c0 + DW;
-  const int nT = (3 - k) * (4 - k) / 2 - 1, nZ = (3 - k) * (k + 1);
+  const int nT = (np - 1 - k) * (np - k) / 2 - 1, nZ = (np - 1 - k) * (k + 1);
   const int nchunks = 2 * (nT + nZ);
   const int wi = t >> 5, lane = t & 31;
 #pragma unroll 1
@@ -477,7 +487,7 @@ __device__ __forceinline__ void diag_panel_update(float2* sS, const float2* Wt, 
       sb = k + 1;
       rb = k + 1;
       while (e > 0) {
-        if (++rb > 3) { ++sb; rb = sb; }
+        if (++rb >= np) { ++sb; rb = sb; }
         --e;
       }
     } else {
@@ -700,103 +710,109 @@ __global__ void __launch_bounds__(NTHR, 1)
     float2* Sa = (T.sidx >= 0) ? Sacc + (int64_t)T.sidx * TB * TB : nullptr;
     const int quarter = warp & 3, half = warp >> 2;
     const int r = quarter * 32 + lane;
-    if (T.flags & TF_UPDATE) {
-      // ------------------------------------------------------------ partial update task
-      // (a paired task: the second tile from the accumulator at ACC2, with its own columns)
-      if (!s_in) wait_k_block(p, T.kseq, task, deadline);
-      for (int u = 0; u < (pair ? 2 : 1); ++u) {
-        TileTask Tu = T;
-        if (u) {
-          Tu.tile = T.tile2;
-          Tu.c0 = T.c0_2;
-          Tu.cv = T.cv2;
-          Tu.sidx = T.sidx2;
-        }
-        float2* Su = (Tu.sidx >= 0) ? Sacc + (int64_t)Tu.sidx * TB * TB : nullptr;
-        const uint32_t acc = u ? ACC2 : ACC1;
-        for (int pass = 0; pass < 2; ++pass) {
-          const int c0 = half * 64 + pass * 32;
-          float vr[32], vi[32];
-          tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + acc + c0, vr);
-          tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + acc + 128 + c0, vi);
-          float4* slot = acc_slot(Su, r, c0);
-          float2 kin[32];
-          load_s_in(Tu, p.K, s_in ? Su : nullptr, r, c0, kin);   // all loads first
-#pragma unroll
-          for (int i = 0; i < 32; i += 2)
-            slot[(i / 2) * TB] = make_float4(kin[i].x - vr[i], kin[i].y - vi[i], kin[i + 1].x - vr[i + 1], kin[i + 1].y - vi[i + 1]);
-        }
-      }
-    } else {
-      // ------------------------------------------------------------ final task
-      if (!s_in) wait_k_block(p, T.kseq, task, deadline);
+    const bool is_upd = (T.flags & TF_UPDATE) != 0;
+    if (!s_in) wait_k_block(p, T.kseq, task, deadline);
+    if (!is_upd && !is_diag && tid == 0) {
       // off-diagonal: prefetch the first two chunks of T_J (B operand of the TRSM product)
-      if (!is_diag && tid == 0) {
-        for (int c = 0; c < 2; ++c) {
-          const uint32_t s = t_load & 1, use = t_load >> 1;
-          if (!mbar_wait(smem_u32(&bar_tempty[s]), (use & 1) ^ 1, deadline)) { failed = true; break; }
-          const uint32_t sb = smem_u32(smem + SMEM_T + s * STAGE_B);
-          const uint32_t fb = smem_u32(&bar_tfull[s]);
-          mbar_expect_tx(fb, STAGE_B);
+      for (int c = 0; c < 2; ++c) {
+        const uint32_t s = t_load & 1, use = t_load >> 1;
+        if (!mbar_wait(smem_u32(&bar_tempty[s]), (use & 1) ^ 1, deadline)) { failed = true; break; }
+        const uint32_t sb = smem_u32(smem + SMEM_T + s * STAGE_B);
+        const uint32_t fb = smem_u32(&bar_tfull[s]);
+        mbar_expect_tx(fb, STAGE_B);
 #pragma unroll
-          for (int q = 0; q < Eng<TF>::NPB; ++q)
-            tma_load_2d(sb + q * PLANE, &mapB, c * KC, T.diag * (int)ROWS + q * 128, fb);
-          ++t_load;
+        for (int q = 0; q < Eng<TF>::NPB; ++q)
+          tma_load_2d(sb + q * PLANE, &mapB, c * KC, T.diag * (int)ROWS + q * 128, fb);
+        ++t_load;
+      }
+    }
+    // ------------------------------------------------------------------ phase 2: S = S_in - acc
+    // One loop for the three kinds of task (the code is long and runs at the rate it is fetched): an update
+    // stores S in the tile's accumulator (a paired one also the second tile's, from the accumulator at
+    // ACC2), a diagonal tile in shared memory, an off-diagonal one as operand planes of the TRSM product.
+    float mx = 0.f;                                 // diagonal tile: max |S|^2 over the real lower triangle
+#pragma unroll 1
+    for (int up = 0; up < (pair ? 4 : 2); ++up) {
+      TileTask Tu = T;
+      float2* Su = Sa;
+      uint32_t acc = ACC1;
+      if (up >= 2) {
+        Tu.c0 = T.c0_2;
+        Tu.cv = T.cv2;
+        Su = (T.sidx2 >= 0) ? Sacc + (int64_t)T.sidx2 * TB * TB : nullptr;
+        acc = ACC2;
+      }
+      const int c0 = half * 64 + (up & 1) * 32;
+      float vr[32], vi[32];
+      if (nchunk > 0) {
+        tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + acc + c0, vr);
+        tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + acc + 128 + c0, vi);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) vr[i] = vi[i] = 0.f;
+      }
+      {
+        float2 kin[32];
+        load_s_in(Tu, p.K, s_in ? Su : nullptr, r, c0, kin);   // all loads first
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          vr[i] = kin[i].x - vr[i];
+          vi[i] = kin[i].y - vi[i];
         }
       }
-
-      // ---------------------------------------------------------------- phase 2: S = S_in - acc
-      if (is_diag) {
+      if (is_upd) {
+        float4* slot = acc_slot(Su, r, c0);
+#pragma unroll
+        for (int i = 0; i < 32; i += 2) slot[(i / 2) * TB] = make_float4(vr[i], vi[i], vr[i + 1], vi[i + 1]);
+      } else if (is_diag) {
+        // the lower triangle; the upper one starts at zero (it accumulates the blocks of X)
         float2* sS = reinterpret_cast<float2*>(smem);   // [128][129]
-        float2* s_d = reinterpret_cast<float2*>(smem + DIAG_AUX);
-        for (int pass = 0; pass < 2; ++pass) {
-          const int c0 = half * 64 + pass * 32;
-          float vr[32], vi[32];
-          if (nchunk > 0) {
-            tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + ACC1 + c0, vr);
-            tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + ACC1 + 128 + c0, vi);
-          } else {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) vr[i] = vi[i] = 0.f;
-          }
-          float2 kin[32];
-          load_s_in(T, p.K, s_in ? Sa : nullptr, r, c0, kin);
-#pragma unroll
-          for (int i = 0; i < 32; ++i) sS[r * LDS + c0 + i] = make_float2(kin[i].x - vr[i], kin[i].y - vi[i]);
+        for (int i = 0; i < 32; ++i) {
+          const bool low = c0 + i <= r;
+          if (low && r < T.rv) mx = fmaxf(mx, vr[i] * vr[i] + vi[i] * vi[i]);
+          sS[r * LDS + c0 + i] = low ? make_float2(vr[i], vi[i]) : make_float2(0.f, 0.f);
         }
+      } else if constexpr (TF) {
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          unsigned char* ch = smem + SMEM_S + (c0 / KC + hh) * STAGE_A;
+          store_smem_plane16_tf32(ch + 0 * PLANE, r, vr + 16 * hh);
+          store_smem_plane16_tf32(ch + 1 * PLANE, r, vi + 16 * hh);
+        }
+      } else {
+        unsigned char* ch = smem + SMEM_S + (c0 / KC) * STAGE_A;
+        store_smem_plane32(ch + 0 * PLANE, ch + 2 * PLANE, r, vr);
+        store_smem_plane32(ch + 1 * PLANE, ch + 3 * PLANE, r, vi);
+      }
+    }
+    if (!is_upd) {
+      if (is_diag) {
+        float2* sS = reinterpret_cast<float2*>(smem);
+        float2* s_d = reinterpret_cast<float2*>(smem + DIAG_AUX);
         tc_fence_before();
         __syncthreads();
         trace_mark(p, task, 1);
-        // max |S| over the real lower triangle (breakdown scale)
-        float mx = 0.f;
-        for (int i = tid; i < TB * TB; i += NTHR) {
-          const int rr = i >> 7, cc = i & 127;
-          if (cc <= rr && rr < T.rv) mx = fmaxf(mx, sqrtf(cabs2(sS[rr * LDS + cc])));
-        }
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (lane == 0) s_red[warp] = mx;
-        __syncthreads();
+        if (lane == 0) s_red[warp] = sqrtf(mx);
         // Unpivoted LDL^T and X = L^{-1}, blocked in panels of DW columns (the diag_* functions)
         {
-          // the upper triangle starts at zero (it accumulates the blocks of X)
-          for (int i = tid; i < TB * TB; i += NTHR) {
-            const int rr = i >> 7, cc = i & 127;
-            if (cc > rr) sS[rr * LDS + cc] = make_float2(0.f, 0.f);
-          }
           float2* Wt = s_d + TB;
           float2* Xd = Wt + DW * WT_LD;                 // [2][DW][XD_LD]
-          __syncthreads();
+          // panels of padding alone are done: a unit diagonal, nothing below it
+          const int np = (T.cv + DW - 1) / DW;
+          if (tid < TB && tid >= np * DW) s_d[tid] = make_float2(1.f, 0.f);
           if (warp < 2) diag_block_2warps(sS, s_d, Xd, 0, warp, lane);
           __syncthreads();
 #pragma unroll 1
-          for (int k = 0; k < TB / DW; ++k) {
+          for (int k = 0; k < np; ++k) {
             float2* Xk = Xd + (k & 1) * DW * XD_LD;
-            diag_panel_solve(sS, s_d, Wt, Xk, k, tid);
-            if (k == TB / DW - 1) break;
+            diag_panel_solve(sS, s_d, Wt, Xk, k, np, tid);
+            if (k == np - 1) break;
             diag_next_block(sS, Wt, k, tid);
             __syncthreads();
             if (warp < 2) diag_block_2warps(sS, s_d, Xd + ((k + 1) & 1) * DW * XD_LD, DW * (k + 1), warp, lane);
-            else diag_panel_update(sS, Wt, Xk, k, tid - 64);
+            else diag_panel_update(sS, Wt, Xk, k, np, tid - 64);
             __syncthreads();
           }
           // D_J (L_JJ and L_JJ^{-1} in complex64 are written after the release, below)
@@ -827,8 +843,11 @@ __global__ void __launch_bounds__(NTHR, 1)
           // stores of the planes: bf16 [T_r, T_i] x [hi, lo] (16 threads per 256-byte plane row) or
           // tf32 [T_r, T_i] (32 threads per 512-byte plane row)
           uint4* Bt = reinterpret_cast<uint4*>(opB + (int64_t)T.tile * ROWS * TB * (TF ? 4 : 2));
-          for (int it = tid; it < TB * 16; it += NTHR) {
-            const int n = it >> 4, c8 = it & 15;
+#pragma unroll 1
+          for (int it = warp; it < TB * 16 / 32; it += NTHR / 32) {
+            // a warp takes 8 rows n by 4 groups of 8 columns: loads of sS[k][n] two to a bank, stores of
+            // whole 64-byte spans
+            const int n = (it >> 2) * 8 + (lane >> 2), c8 = (it & 3) * 4 + (lane & 3);
             const float2 dinv = cdiv(make_float2(1.f, 0.f), s_d[n]);
             float tr[8], ti[8];
 #pragma unroll
@@ -862,39 +881,6 @@ __global__ void __launch_bounds__(NTHR, 1)
         __syncthreads();
         trace_mark(p, task, 3);
       } else {
-        // S planes for the TRSM product (A operand, SW64 K-major, 4 chunks)
-        for (int pass = 0; pass < 2; ++pass) {
-          const int c0 = half * 64 + pass * 32;
-          float vr[32], vi[32];
-          if (nchunk > 0) {
-            tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + ACC1 + c0, vr);
-            tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + ACC1 + 128 + c0, vi);
-          } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) vr[i] = vi[i] = 0.f;
-          }
-          {
-            float2 kin[32];
-            load_s_in(T, p.K, s_in ? Sa : nullptr, r, c0, kin);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              vr[i] = kin[i].x - vr[i];
-              vi[i] = kin[i].y - vi[i];
-            }
-          }
-          if constexpr (TF) {
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-              unsigned char* ch = smem + SMEM_S + (c0 / KC + hh) * STAGE_A;
-              store_smem_plane16_tf32(ch + 0 * PLANE, r, vr + 16 * hh);
-              store_smem_plane16_tf32(ch + 1 * PLANE, r, vi + 16 * hh);
-            }
-          } else {
-            unsigned char* ch = smem + SMEM_S + (c0 / KC) * STAGE_A;
-            store_smem_plane32(ch + 0 * PLANE, ch + 2 * PLANE, r, vr);
-            store_smem_plane32(ch + 1 * PLANE, ch + 3 * PLANE, r, vi);
-          }
-        }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
         __syncthreads();
@@ -946,6 +932,7 @@ __global__ void __launch_bounds__(NTHR, 1)
         float2* s_d = reinterpret_cast<float2*>(smem + SMEM_T);
         if (tid < TB) s_d[tid] = ld_cg(Dg + (int64_t)T.col * TB + tid);
         float4* stg = reinterpret_cast<float4*>(smem);
+#pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
           const int c0 = half * 64 + pass * 32;
           float lr[32], li[32];
@@ -963,6 +950,7 @@ __global__ void __launch_bounds__(NTHR, 1)
         // (read only by the solve sweeps) is written after the release, below
         uint4* A = reinterpret_cast<uint4*>(opA + (int64_t)T.tile * ROWS * TB * (TF ? 4 : 2));
         uint4* B = reinterpret_cast<uint4*>(opB + (int64_t)T.tile * ROWS * TB * (TF ? 4 : 2));
+#pragma unroll 1
         for (int it = tid; it < TB * 16; it += NTHR) {
           const int rr = it >> 4, c8 = it & 15;   // row, group of 8 columns
           float2 l[8];
