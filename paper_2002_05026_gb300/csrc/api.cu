@@ -614,7 +614,7 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
       for (int k : l)
         for (int I = S.tstart[k]; I < S.tstart[k + 1]; ++I) {
           mf = std::max<int64_t>(mf, S.fwd_slot_ptr[I] >> 32);
-          mb = std::max<int64_t>(mb, (S.bwd_slot_ptr[I] >> 32) * (b / 64));
+          mb = std::max<int64_t>(mb, S.bwd_slot_ptr[I] >> 32);
         }
       h->lev_maxcnt_fwd.push_back((int32_t)mf);
       h->lev_maxcnt_bwd.push_back((int32_t)mb);

@@ -4,9 +4,9 @@
 // with the source vectors already solved (Sec. II: the solution phase runs over the same block
 // tasks as the factorization):
 //   forward   P[slot][r][j]   = sum_items sum_c L_IJ[r][c] y_J[c][j]      (destination row tile I)
-//   backward  P[slot][0][c][j] = sum_items sum_r L_IJ[r][c] w_I[r][j]     (destination column tile J)
-// in the partial layout of the SIMT gather (backward: the whole sum in sub-slot 0, zeros in the
-// others), so the block chains that consume the partials are unchanged.
+//   backward  P[slot][c][j]   = sum_items sum_r L_IJ[r][c] w_I[r][j]     (destination column tile J)
+// in the partial layout of the SIMT gather's forward direction (one sub-slot of 128 rows per slot, where
+// the SIMT backward gather fills one per 64 rows of the tiles).
 //
 // Arithmetic: split-BF16x3 products (a = hi + lo; hi*hi + hi*lo + lo*hi) accumulated in FP32 in
 // tensor memory, the same operands and accuracy as the factorization's tile engine.  The L tiles
@@ -267,20 +267,21 @@ __global__ void __launch_bounds__(GTH, 1)
       const uint32_t buf = un & 1, ause = un >> 1;
       if (!gbar_wait(su32g(&acc_full[buf]), ause & 1, deadline)) { ok = false; break; }
       gfence_after();
-      float2* out = FWD ? P + (int64_t)g.slot * nh * b * nrhs + (int64_t)row * nrhs
-                        : P + (int64_t)g.slot * nh * b * nrhs + (int64_t)row * nrhs;
+      float2* out = P + ((int64_t)g.slot * nh * b + row) * nrhs + j0;
+      const bool wide = ((nrhs | j0) & 1) == 0;  // two right-hand sides a store
       for (int jb = 0; jb < NR; jb += 8) {
         float re[8], im[8];
         gtmem_ld8(tmem + ((uint32_t)(quad * 32) << 16) + buf * GACC + jb, re);
         gtmem_ld8(tmem + ((uint32_t)(quad * 32) << 16) + buf * GACC + NR + jb, im);
+        if (wide) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (j0 + jb + q < nrhs) out[j0 + jb + q] = make_float2(re[q], im[q]);
-      }
-      if (!FWD) {
-        // the other 64-row sub-slot of the backward partial holds zeros
-        float2* z = P + ((int64_t)g.slot * nh + 1) * b * nrhs + (int64_t)row * nrhs;
-        for (int q = 0; q < NR && j0 + q < nrhs; ++q) z[j0 + q] = make_float2(0.f, 0.f);
+          for (int q = 0; q < 8; q += 2)
+            if (j0 + jb + q < nrhs) *reinterpret_cast<float4*>(out + jb + q) = make_float4(re[q], im[q], re[q + 1], im[q + 1]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (j0 + jb + q < nrhs) out[jb + q] = make_float2(re[q], im[q]);
+        }
       }
       gfence_before();
       __syncwarp();

@@ -39,7 +39,7 @@ struct SweepLaunch {
   const int64_t* tcolptr;          // device [NT+1]
   const int32_t* lev_maxnt;        // host [nlevels]: most tiles of one block in the level
   const int32_t* lev_maxcnt_fwd;   // host [nlevels]: most forward partials of one tile row
-  const int32_t* lev_maxcnt_bwd;   // host [nlevels]: most backward partials of one tile column
+  const int32_t* lev_maxcnt_bwd;   // host [nlevels]: most backward partial slots of one tile column
   const void* Inv;                 // off-diagonal tiles of the diagonal blocks' inverses, or nullptr
   const int* done;                 // device [instances]: converged instances are skipped, or nullptr
   const int32_t* tinst;            // device [NT]: instance of every tile row (permuted numbering)

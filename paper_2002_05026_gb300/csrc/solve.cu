@@ -965,6 +965,7 @@ struct ChainSweep {
   int b, nrhs, rc;           // rhs per cluster (grid.y = ceil(nrhs / rc))
   int cl, nloc, stg;         // CTAs per cluster, strip slots per CTA, elements of one stage buffer
   int has_partials;
+  int nsub;                  // partials per slot (SIMT backward gather: one per 64 rows of a tile, else 1)
   int apply_d;               // backward: divide the loaded strips by D (else a reduce launch did)
   Mask mk;
   const void* Inv;           // off-diagonal tiles of the inverses of the diagonal blocks (INV mode)
@@ -977,7 +978,10 @@ struct ChainSweep {
 constexpr int CHAIN_MAXJ = 128;   // staged strips of one CTA
 constexpr int CHAIN_MAXCL = 8;    // portable cluster size
 constexpr int CHAIN_MAXLOC = 4;   // strips per CTA
-constexpr int EXT_REDUCE = 12;    // partials per row above which a level gets a separate reduce launch
+// Partials per row above which a level gets a separate reduce launch: the chain subtracts fewer itself, sixteen
+// loads in flight a thread, in less time than a launch takes (at 12: 6.3 ms of sweeps on a 5 x 5 x 3 grid, m = 256,
+// 32 right-hand sides, at 80 6.0 ms; 8 x 8, m = 512: 3.82, 3.78 at 32, 3.85 at 80).
+constexpr int EXT_REDUCE = 48;
 
 // INV mode: the diagonal block is applied as one product with its stored inverse,
 //   y_J = L_JJ^{-1} r_J (forward),  w_J = L_JJ^{-T} r_J (backward),
@@ -1080,9 +1084,9 @@ __global__ void __launch_bounds__(GT) chain_kernel(ChainSweep s, const typename 
       if (s.has_partials) {
         const int64_t sp = s.slot_ptr[I];
         first = sp & 0xffffffffLL;
-        cnt = (sp >> 32) * (FWD ? 1 : nh);
+        cnt = (sp >> 32) * s.nsub;
       }
-      const int64_t stride = (int64_t)b * s.nrhs * (FWD ? nh : 1);
+      const int64_t stride = (int64_t)b * s.nrhs * (s.nsub == 1 ? nh : 1);
       for (int i = threadIdx.x; i < HR * rc; i += GT) {
         const int j = i % rc, row = i / rc;
         const int64_t g = (int64_t)I * b + h * HR + row;
@@ -1396,15 +1400,14 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
   // Right-hand sides per block: the products run over a compile-time count RC (a power of two), so that
   // few right-hand sides do not pay for eight.  FP64 products are bound by the FP64 pipe (a 64 x 64 tile
   // times 8 right-hand sides holds an SM for 43 us), so there the right-hand sides are also spread over
-  // more blocks while a level leaves SMs idle; FP32 ones are bound by the tile's loads, which that would
-  // repeat.  FP64 sweeps of a 4 x 4 grid, m = 512, 8 right-hand sides: 13.8 -> 7.7 ms; 3 x 3, m = 100, 3
+  // more blocks while a level leaves SMs idle.  So they are in the chains of either type, whose time is the
+  // latency of one block's steps; FP32 gathers are bound by the tile's loads, which that would repeat.  FP64 sweeps of a 4 x 4 grid, m = 512, 8 right-hand sides: 13.8 -> 7.7 ms; 3 x 3, m = 100, 3
   // right-hand sides: 2.4 -> 0.54 ms; complex64, 8 x 8, m = 256, 1 right-hand side: 3.3 -> 2.8 ms.
   int rmax = 1;
   while (rmax < a.nrhs && rmax < RCMAX) rmax <<= 1;
-  const int64_t nsm_rc = sizeof(R) == 8 ? a.nsm : 0;
   auto pick_rc = [&](int64_t blocks) {
     int rc = rmax;
-    while (rc > 1 && blocks * ((a.nrhs + rc / 2 - 1) / (rc / 2)) <= nsm_rc) rc >>= 1;
+    while (rc > 1 && blocks * ((a.nrhs + rc / 2 - 1) / (rc / 2)) <= a.nsm) rc >>= 1;
     return rc;
   };
   int nsm = 0;
@@ -1422,7 +1425,7 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
       return;
     }
     const int nunits = (int)((i1 - i0) * nh);
-    const int rc = pick_rc(nunits);
+    const int rc = sizeof(R) == 8 ? pick_rc(nunits) : rmax;
     with_rc(rc, [&](auto k) {
       constexpr int RC = decltype(k)::value;
       auto kern = fwd ? gather_kernel<R, true, RC> : gather_kernel<R, false, RC>;
@@ -1470,6 +1473,8 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
     cs.invT_off = a.invT_off;
     cs.mk = mk;
     cs.rrows = (int)rrows;
+    // partials per slot of a backward gather
+    const int bsub = a.tcmaps && sizeof(R) == 4 ? 1 : nh;
     auto launch_chain = [&](int lv, bool fwd) -> cudaError_t {
       const int S = a.lev_maxnt[lv] * nh;
       cs.cl = std::min(CHAIN_MAXCL, S);
@@ -1513,6 +1518,7 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
       }
       cs.slot_ptr = a.fwd_slot_ptr;
       cs.has_partials = i1 > i0;
+      cs.nsub = 1;
       cs.apply_d = 0;
       if (i1 > i0 && a.lev_maxcnt_fwd[lv] > EXT_REDUCE) {
         // many partials per row: a wide reduce launch is cheaper than the cluster's strip loads
@@ -1540,12 +1546,13 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
       }
       cs.slot_ptr = a.bwd_slot_ptr;
       cs.has_partials = i1 > i0;
+      cs.nsub = bsub;
       cs.apply_d = bk ? 0 : 1;
-      if (i1 > i0 && a.lev_maxcnt_bwd[lv] > EXT_REDUCE) {
+      if (i1 > i0 && a.lev_maxcnt_bwd[lv] * bsub > EXT_REDUCE) {
         const int64_t ntl = a.lev_tile_ptr[lv + 1] - a.lev_tile_ptr[lv];
         const int64_t nthr = ntl * b * a.nrhs;
         launch_pdl(reduce_kernel<R>, dim3((unsigned)((nthr + 31) / 32)), dim3(ET), 0, st, a.lev_tiles + a.lev_tile_ptr[lv], (int)ntl,
-                                                                       a.bwd_slot_ptr, P, Y, a.npad, b, a.nrhs, nh, bk ? nullptr : D, mk);
+                                                                       a.bwd_slot_ptr, P, Y, a.npad, b, a.nrhs, bsub, bk ? nullptr : D, mk);
         ++a.launches;
         cs.has_partials = 0;
         cs.apply_d = 0;
@@ -1603,7 +1610,7 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
       launch_gather(false, i0, i1);
       const int64_t nthr = ntl * b * a.nrhs;
       launch_pdl(reduce_kernel<R>, dim3((unsigned)((nthr + 31) / 32)), dim3(ET), 0, st, a.lev_tiles + a.lev_tile_ptr[lv], (int)ntl,
-                                                                     a.bwd_slot_ptr, P, Y, a.npad, b, a.nrhs, nh, nullptr, mk);
+                                                                     a.bwd_slot_ptr, P, Y, a.npad, b, a.nrhs, a.tcmaps && sizeof(R) == 4 ? 1 : nh, nullptr, mk);
       a.launches += 2;
     }
     bs.blocks = a.lev_blocks + a.lev_ptr[lv];

@@ -573,8 +573,11 @@ int analyze(const d3m_pattern* pat, const int32_t* perm_in, int b, bool build_ta
       int64_t e1 = e;
       while (e1 < i1 && items[e1].dst == d) ++e1;
       const int64_t first_slot = (int64_t)groups.size() - g0;
-      for (int64_t q = e; q < e1; q += G) {
-        const int32_t cnt = (int32_t)std::min<int64_t>(G, e1 - q);
+      // equal shares (they differ by one item at most)
+      const int64_t n = e1 - e, ng = (n + G - 1) / G;
+      for (int64_t u = 0; u < ng; ++u) {
+        const int64_t q = e + n * u / ng;
+        const int32_t cnt = (int32_t)(e + n * (u + 1) / ng - q);
         groups.push_back(SolveGroup{(int32_t)q, cnt, (int32_t)((int64_t)groups.size() - g0), d});
         s.max_group = std::max(s.max_group, cnt);
       }
@@ -582,6 +585,8 @@ int analyze(const d3m_pattern* pat, const int32_t* perm_in, int b, bool build_ta
       slot_ptr[d] = first_slot | (nslot << 32);
       e = e1;
     }
+    // the blocks of a gather take groups i, i + grid, ...: the longest first
+    std::stable_sort(groups.begin() + g0, groups.end(), [](const SolveGroup& a, const SolveGroup& c) { return a.count > c.count; });
     return (int64_t)groups.size() - g0;
   };
   for (int lv = 0; lv < s.nlevels; ++lv) {
