@@ -31,7 +31,7 @@
  *     loop inside d3m_solve, which reads one convergence word per iteration.
  *
  * Ownership: the caller owns every buffer it passes and the stream.  The library owns the
- * factors, the base-64 digit planes of K (kept for the FP64-accurate residual), a copy buffer for a host K
+ * factors, the base-32 digit planes of K (kept for the FP64-accurate residual), a copy buffer for a host K
  * (allocated by the first d3m_factor that passes one), the task graph and its workspaces, from
  * d3m_create until d3m_destroy.  A handle is not thread-safe; use one per host thread.
  *

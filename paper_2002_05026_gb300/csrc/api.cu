@@ -129,7 +129,6 @@ struct d3m_ctx {
   double2* contract = nullptr;
   // FP64-accurate residual on the tensor cores: digit planes of K (per factorization) and x
   ResidualTc rtc{};
-  ResidTcMaps rtc_maps;
   std::vector<int2> rtile_host;      // (row block f, 128-row tile)
   int max_rtiles = 1;
   // batched handles: independent systems stored as one block-diagonal system
@@ -684,8 +683,8 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
   UPLOAD(h->res_tr, S.res_tr);
   {
     // residual digit planes: per contribution e of row block f from block g, ceil(m_f / 128) row
-    // tiles x ceil(m_g / 32) chunks x 2 parts x 9 digits planes of 128 x 32 bf16; per block g,
-    // ceil(m_g / 32) chunks x 2 x 9 planes of 64 x 32 bf16 for the digits of x
+    // tiles x ceil(m_g / 32) chunks x 2 parts x 11 digits planes of 128 x 32 e4m3; per block g,
+    // ceil(m_g / 32) chunks x 2 x 11 planes of 32 x 32 e4m3 for the digits of x
     const int64_t nres = (int64_t)S.res_blk.size();
     std::vector<int64_t> ksp(nres), xsp(S.N);
     std::vector<int32_t> rrow(nres), brow(S.nnzb_K), bcol(S.nnzb_K);
@@ -742,14 +741,12 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
     // an FP64 solve without omega never forms a residual
     h->resid = !h->fp64 || h->opt.fp64_omega != 0;
     if (h->resid) {
-      ALLOC(r.kdig, unsigned short, pa * 128 * 32);
-      ALLOC(r.xdig, unsigned short, pb * ngrp * 64 * 32);
+      ALLOC(r.kdig, unsigned char, pa * 128 * 32);
+      ALLOC(r.xdig, unsigned char, pb * ngrp * 32 * 32);
       ALLOC(r.Kmax_bits, unsigned long long, S.nnzb_K);
       ALLOC(r.Kdiag, double2, S.n);
       ALLOC(r.rowsum, float, S.n);
       ALLOC(r.xT, int, (size_t)ngrp * S.N * 32);
-      std::string e3;
-      if (resid_tc_make_maps(r.kdig, pa, r.xdig, pb * ngrp, &h->rtc_maps, e3) != 0) return set_err(h, D3M_ERR_CUDA, e3);
     }
   }
   UPLOAD(h->m_orig, S.m_orig);
@@ -1101,7 +1098,7 @@ static int residual_omega(d3m_ctx* h, const double2* X, const double2* B, int nr
   ResidualTc rp = resid_params(h, nullptr);
   ev_begin(h, d3m_ctx::EV_RESID, st);
   int64_t nl = 0;
-  int rc = launch_resid_tc(rp, h->rtc_maps, X, B, h->d_r, nrhs, (int)h->rtile_host.size(), h->S.N, st, &nl);
+  int rc = launch_resid_tc(rp, X, B, h->d_r, nrhs, (int)h->rtile_host.size(), h->S.N, h->max_rtiles, st, &nl);
   if (rc) return set_err(h, D3M_ERR_CUDA, std::string("residual launch: ") + cudaGetErrorString((cudaError_t)rc));
   ev_end(h, d3m_ctx::EV_RESID, st);
   h->launches += nl;

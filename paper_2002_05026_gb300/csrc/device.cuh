@@ -105,6 +105,39 @@ __device__ __forceinline__ float2 cdiv(float2 a, float2 b) {
 __device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
 __device__ __forceinline__ float cabs2(float2 a) { return a.x * a.x + a.y * a.y; }
 
+// (hi 2^LB + lo) 2^e rounded to FP64 (nearest; underflow to zero, overflow to infinity).  Integer
+// instructions only: conversions and adds on the FP64 pipe (64 cycles a warp and SM partition each) would
+// take longer than the products that the sums come from.
+template <int LB>
+__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int e) {
+  hi += lo >> LB;
+  uint32_t l = (uint32_t)lo & ((1u << LB) - 1);    // value = hi 2^LB + l, 0 <= l < 2^LB
+  const bool neg = hi < 0;
+  unsigned long long h = (unsigned long long)hi;
+  if (neg) {
+    h = l ? ~h : 0ull - h;
+    l = l ? (1u << LB) - l : 0u;
+  }
+  int lz = __clzll((long long)h);
+  unsigned long long m;                            // top bit at 63
+  if (lz < LB) {
+    m = (h << lz) | (unsigned long long)(l >> (LB - lz));
+    e += LB + 63 - lz;
+  } else {
+    const unsigned long long x = (h << LB) | l;
+    if (x == 0) return 0.0;
+    lz = __clzll((long long)x);
+    m = x << lz;
+    e += 63 - lz;
+  }
+  const unsigned long long r = (m >> 11) + ((m >> 10) & 1);   // 53 bits; 2^53 carries into the exponent
+  const int be = e + 1023;
+  unsigned long long bits = ((unsigned long long)(be - 1) << 52) + r;
+  if (be <= 0) bits = 0;
+  else if (be >= 2047) bits = 0x7ffull << 52;
+  return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
+}
+
 template <typename R> struct CT;
 template <> struct CT<double> {
   using C = double2;

@@ -248,37 +248,6 @@ __device__ __forceinline__ void put_digits(unsigned char* st, bool w_side, int r
   }
 }
 
-// (hi 2^28 + lo) 2^e rounded to FP64 (nearest; underflow to zero, overflow to infinity).  Integer
-// instructions only: conversions and adds on the FP64 pipe would take longer than the products.
-__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int e) {
-  hi += lo >> 28;
-  uint32_t l = (uint32_t)lo & 0x0fffffffu;         // value = hi 2^28 + l, 0 <= l < 2^28
-  const bool neg = hi < 0;
-  unsigned long long h = (unsigned long long)hi;
-  if (neg) {
-    h = l ? ~h : 0ull - h;
-    l = l ? 0x10000000u - l : 0u;
-  }
-  int lz = __clzll((long long)h);
-  unsigned long long m;                            // top bit at 63
-  if (lz < 28) {
-    m = (h << lz) | (unsigned long long)(l >> (28 - lz));
-    e += 28 + 63 - lz;
-  } else {
-    const unsigned long long x = (h << 28) | l;
-    if (x == 0) return 0.0;
-    lz = __clzll((long long)x);
-    m = x << lz;
-    e += 63 - lz;
-  }
-  const unsigned long long r = (m >> 11) + ((m >> 10) & 1);   // 53 bits; 2^53 carries into the exponent
-  const int be = e + 1023;
-  unsigned long long bits = ((unsigned long long)(be - 1) << 52) + r;
-  if (be <= 0) bits = 0;
-  else if (be >= 2047) bits = 0x7ffull << 52;
-  return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
-}
-
 // x 2^k by its exponent field (zero and what leaves the range of normal numbers: 0)
 __device__ __forceinline__ double scale2(double x, int k) {
   const long long u = __double_as_longlong(x);
@@ -524,7 +493,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
     };
     auto result = [&](int i) -> double {
       if (max(s_MA[r0 + i], s_MB[oc]) >= E_BAD) return __longlong_as_double(0x7ff8000000000000ll);
-      return fixed_to_double(H[i], Lo[i], s_MA[r0 + i] + s_MB[oc] - 74);
+      return fixed_to_double<28>(H[i], Lo[i], s_MA[r0 + i] + s_MB[oc] - 74);
     };
 
     // ---------------------------------------------------------------- 1. Schur products
@@ -754,7 +723,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
 #pragma unroll
           for (int i = 0; i < 4; ++i)
             sV[(ri * TB + oc) * (PW + 1) + q0 + i] =
-                m >= E_BAD ? __longlong_as_double(0x7ff8000000000000ll) : fixed_to_double(H[i], Lo[i], s_MA[q0 + i] + s_MB[oc] - 74);
+                m >= E_BAD ? __longlong_as_double(0x7ff8000000000000ll) : fixed_to_double<28>(H[i], Lo[i], s_MA[q0 + i] + s_MB[oc] - 74);
         }
         __syncthreads();
         // above the panel X = -V, below L = V / d
@@ -785,7 +754,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
               const int r = rb + i;
               if (oc <= r) {
                 const double v = max(s_MA[r], s_MB[oc]) >= E_BAD ? __longlong_as_double(0x7ff8000000000000ll)
-                                                                   : fixed_to_double(H[i], Lo[i], s_MA[r] + s_MB[oc] - 74);
+                                                                   : fixed_to_double<28>(H[i], Lo[i], s_MA[r] + s_MB[oc] - 74);
                 double* t = reinterpret_cast<double*>(oc >= c1 ? sS + r * LDS + oc : sS + oc * LDS + r) + ri;
                 *t -= v;
               }

@@ -66,7 +66,7 @@ int launch_gather_tc(bool fwd, const GatherTcMaps& maps, const SolveGroup* group
                      const int32_t* tinst, int nunits, int nsm, cudaStream_t st);
 
 // FP64-accurate residual on the tensor cores (resid_tc.cu): digit planes of K and x.
-constexpr int kResidDigits = 9;       // base-64 digits per value; 2 x kResidDigits planes per chunk
+constexpr int kResidDigits = 11;      // base-32 digits per value; 2 x kResidDigits planes per chunk
 struct ResidualTc {
   const double2* K;              // stored lower blocks (c128), read by the digit kernels only
   const int64_t* kblk_off;       // [nnzb+1]
@@ -86,8 +86,8 @@ struct ResidualTc {
   int64_t xs_total;              // x digit planes of one right-hand-side group
   int nblk;                      // N
   const int2* rtiles;            // [row tiles] (row block f, 128-row tile)
-  unsigned short* kdig;          // K digit planes (bf16), 128 x 32 each
-  unsigned short* xdig;          // x digit planes (bf16), 64 x 32 each
+  unsigned char* kdig;           // K digit planes (e4m3), 128 x 32 each
+  unsigned char* xdig;           // x digit planes (e4m3), 32 x 32 each
   unsigned long long* Kmax_bits; // [nnzb] max |Re|, |Im| of every stored block (double bits)
   double2* Kdiag;                // [n] diagonal entries of K (applied in FP64)
   float* rowsum;                 // [n] row sums of |K| (for ||K||_inf)
@@ -104,17 +104,10 @@ struct ResidualTc {
   int64_t timeout_ns;
 };
 
-struct ResidTcMaps {
-  alignas(64) unsigned char a[128];
-  alignas(64) unsigned char b[4][128];
-};
-
-int resid_tc_make_maps(void* kdig, int64_t nplanes_a, void* xdig, int64_t nplanes_b, ResidTcMaps* out,
-                       std::string& err);
 int launch_kdigits(const ResidualTc& p, int nnzb, int nres, int max_rtiles, int nblk, cudaStream_t st);
 int resid_tc_groups(int nrhs, int* NR);
-int launch_resid_tc(const ResidualTc& p, const ResidTcMaps& maps, const double2* X, const double2* B, double2* R,
-                    int nrhs, int nrtiles, int nblk, cudaStream_t st, int64_t* launches);
+int launch_resid_tc(const ResidualTc& p, const double2* X, const double2* B, double2* R,
+                    int nrhs, int nrtiles, int nblk, int max_rtiles, cudaStream_t st, int64_t* launches);
 
 // Tensor maps (CUtensorMap, 128 bytes each) of the tensor-core operand planes.
 struct TcMaps {
