@@ -47,6 +47,9 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ------------------------------------------------------------------ permutation + padding
+// Row blocks of 256 by groups of PERM_RC right-hand sides, whose loads are in flight together.  32 right-hand sides
+// of 43,000 rows: in 16 -> 10 us, out 60 -> 17 us against one thread for all of a row's right-hand sides.
+constexpr int PERM_RC = 4, PERM_WARPS = 8;
 template <typename R>
 __global__ void permute_in_kernel(const double2* __restrict__ src, int64_t n,
                                   typename CT<R>::C* __restrict__ Y, int64_t npad,
@@ -56,12 +59,17 @@ __global__ void permute_in_kernel(const double2* __restrict__ src, int64_t n,
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (g >= npad || mk.off(g / b)) return;
   const int64_t o = pad2orig[g];
-  for (int j = 0; j < nrhs; ++j)
+  const int j1 = min(nrhs, ((int)blockIdx.y + 1) * PERM_RC);
+#pragma unroll PERM_RC
+  for (int j = blockIdx.y * PERM_RC; j < j1; ++j)
     Y[j * npad + g] = (o >= 0) ? CT<R>::from(src[j * n + o]) : CT<R>::make(0, 0);
 }
 
 // X (=, or += when accumulate) W in caller numbering; dmax[instance * ld + j] = max |W| of the
-// step (float bits; the size of the correction drives the forward-error stopping test).
+// step (float bits; the size of the correction drives the forward-error stopping test).  |W|^2 is formed
+// in FP32 with the rounding errors of its products and its sum added back (as close as an FP64 sum rounded to
+// FP32: the FP64 pipe holds a warp 64 cycles an instruction, and only the update itself needs it).  A block joins
+// its warps' maxima: one atomic a warp and right-hand side, all on one line of L2, took most of the time.
 template <typename R>
 __global__ void permute_out_kernel(const typename CT<R>::C* __restrict__ W, int64_t npad,
                                    double2* __restrict__ X, int64_t n,
@@ -70,17 +78,26 @@ __global__ void permute_out_kernel(const typename CT<R>::C* __restrict__ W, int6
   pdl_trigger();
   pdl_wait();
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g - (threadIdx.x & 31) >= npad) return;              // whole warps past the end
+  __shared__ unsigned s_max[PERM_RC][PERM_WARPS];
+  __shared__ int s_inst[PERM_WARPS];
   // a warp's 32 rows lie in one tile (tiles are >= 64 rows and warps 32-aligned)
   const bool act = g < npad && !mk.off(g / b) && pad2orig[g] >= 0;   // a converged instance keeps its x
   const int64_t o = act ? pad2orig[g] : 0;
   const int inst = (g < npad && mk.tinst) ? mk.tinst[g / b] : 0;
-  for (int j = 0; j < nrhs; ++j) {
+  const int j1 = min(nrhs, ((int)blockIdx.y + 1) * PERM_RC);
+#pragma unroll PERM_RC
+  for (int j = blockIdx.y * PERM_RC; j < j1; ++j) {
     float a = 0.f;
     if (act) {
       const typename CT<R>::C w = W[j * npad + g];
       double2 v = make_double2((double)w.x, (double)w.y);
-      a = sqrtf((float)(v.x * v.x + v.y * v.y));
+      if constexpr (sizeof(R) == 4) {
+        const float p = w.x * w.x, q = w.y * w.y, s = p + q, z = s - p;
+        const float e = fmaf(w.x, w.x, -p) + fmaf(w.y, w.y, -q) + ((p - (s - z)) + (q - z));
+        a = sqrtf(s < 3.0e38f ? s + e : s);
+      } else {
+        a = sqrtf((float)(v.x * v.x + v.y * v.y));
+      }
       if (accumulate) {
         const double2 x = X[j * n + o];
         v.x += x.x;
@@ -88,8 +105,22 @@ __global__ void permute_out_kernel(const typename CT<R>::C* __restrict__ W, int6
       }
       X[j * n + o] = v;
     }
-    for (int s = 16; s > 0; s >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, s));
-    if (dmax && (threadIdx.x & 31) == 0 && a > 0.f) atomicMax(dmax + inst * ld + j, __float_as_uint(a));
+    const unsigned w = __reduce_max_sync(0xffffffffu, a > 0.f ? __float_as_uint(a) : 0u);   // a NaN counts as 0
+    if ((threadIdx.x & 31) == 0) s_max[j & (PERM_RC - 1)][threadIdx.x >> 5] = w;
+  }
+  if (!dmax) return;
+  if ((threadIdx.x & 31) == 0) s_inst[threadIdx.x >> 5] = inst;
+  __syncthreads();
+  const int j = blockIdx.y * PERM_RC + threadIdx.x;
+  if (threadIdx.x < PERM_RC && j < j1) {
+    unsigned m = 0;
+#pragma unroll
+    for (int w = 0; w < PERM_WARPS; ++w) {
+      m = max(m, s_max[threadIdx.x][w]);
+      if (w + 1 < PERM_WARPS && s_inst[w + 1] == s_inst[w]) continue;
+      if (m) atomicMax(dmax + s_inst[w] * ld + j, m);
+      m = 0;
+    }
   }
 }
 
@@ -1241,28 +1272,36 @@ __global__ void vec_absmax_kernel(const double2* __restrict__ V, int64_t n, int 
 // omega_(i,j) = |r|_(i,j) / (||K_i|| |x|_(i,j) + |b|_(i,j)) for instance i, column j (entry
 // i * ld + j), recomputed for the instances still refining (a converged instance keeps the values
 // of the step that converged it, and done[i] is set once all its columns meet tol);
-// stat[0] = the largest over all instances.  One block of 256 threads.
+// stat[0] = the largest over all instances.
 // An instance is done when every column has omega <= tol and a small forward error: the last
 // correction d_k is at most ftol of |x|, or, with the contraction rho = |d_k| / |d_(k-1)| < 1,
 // the error left in x (about rho / (1 - rho) |d_k|) is (ftol <= 0 skips the forward test).
 // stat[0] = the largest omega, stat[1] = instances not done.
+// One block of 256 threads; `width` (a power of two <= 32) lanes share an instance and take its columns in
+// turn.  Bound by the latency of its FP64 divisions: one thread an instance took 85 us for 32 columns, a lane a
+// column 7 us.
 __global__ void omega_kernel(const unsigned* rmax, const unsigned* xmax, const unsigned* bmax,
                              const unsigned* kmax, const unsigned* dmax, float* dprev, int ninst, int ld,
-                             int nrhs, int* done, double tol, double ftol, double* omega, double* stat) {
+                             int nrhs, int width, int* done, double tol, double ftol, double* omega, double* stat) {
   double w = 0.0, mu = 0.0;   // mu: how far the open instances are from both targets
   int open = 0;
-  for (int i = threadIdx.x; i < ninst; i += blockDim.x) {
-    double wi = 0.0, mui = 0.0;
-    if (!done[i]) {
+  const int sub = threadIdx.x & (width - 1), per = blockDim.x / width;
+  for (int i0 = 0; i0 < ninst; i0 += per) {
+    const int i = i0 + threadIdx.x / width;
+    const bool there = i < ninst, was = there && done[i];
+    bool ok = true;
+    double mui = 0.0;
+    if (was) {
+      for (int j = sub; j < nrhs; j += width) w = fmax(w, omega[i * ld + j]);
+    } else if (there) {
       const double kn = (double)__uint_as_float(kmax[i]);
-      bool ok = true;
-      for (int j = 0; j < nrhs; ++j) {
+      for (int j = sub; j < nrhs; j += width) {
         const int q = i * ld + j;
         const double r = __uint_as_float(rmax[q]), x = __uint_as_float(xmax[q]), bb = __uint_as_float(bmax[q]);
         const double den = kn * x + bb;
         const double o = den > 0 ? r / den : (r > 0 ? 1.0 : 0.0);
         omega[q] = o;
-        wi = fmax(wi, o);
+        w = fmax(w, o);
         const double d = __uint_as_float(dmax[q]), dp = dprev[q];
         const double ratio = x > 0 ? d / x : (d > 0 ? 1.0 : 0.0);
         const double rho = dp > 0 ? d / dp : 1.0;
@@ -1271,15 +1310,18 @@ __global__ void omega_kernel(const unsigned* rmax, const unsigned* xmax, const u
         mui = fmax(mui, fmax(o / tol, ftol > 0 ? ratio / ftol : 0.0));
         dprev[q] = (float)d;
       }
-      if (ok) done[i] = 1;
-      else {
-        ++open;
+    }
+    // the instance's lanes agree (all threads of the block are here)
+    int all = ok;
+    for (int o = width / 2; o > 0; o >>= 1) all &= __shfl_xor_sync(0xffffffffu, all, o);
+    if (there && !was) {
+      if (all) {
+        if (sub == 0) done[i] = 1;
+      } else {
+        if (sub == 0) ++open;
         mu = fmax(mu, mui);
       }
-    } else {
-      for (int j = 0; j < nrhs; ++j) wi = fmax(wi, omega[i * ld + j]);
     }
-    w = fmax(w, wi);
   }
   __shared__ double s_w[256], s_mu[256];
   __shared__ int s_o[256];
@@ -1380,8 +1422,9 @@ template <typename R>
 static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
   using C = typename CT<R>::C;
   const int b = a.b;
-  const int nthreads = 256;
+  const int nthreads = 32 * PERM_WARPS;
   const int64_t gblocks = (a.npad + nthreads - 1) / nthreads;
+  const dim3 pgrid((unsigned)gblocks, (unsigned)((a.nrhs + PERM_RC - 1) / PERM_RC));
   const C* L = (const C*)a.L;
   const C* Linv = (const C*)a.Linv;
   const C* D = (const C*)a.D;
@@ -1390,7 +1433,7 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
   const int nh = b / HR;
   a.launches = 0;
   const Mask mk{a.done, a.tinst};
-  launch_pdl(permute_in_kernel<R>, dim3((unsigned)gblocks), dim3(nthreads), 0, st, a.src, a.n, Y, a.npad, a.pad2orig, a.nrhs, mk, b);
+  launch_pdl(permute_in_kernel<R>, pgrid, dim3(nthreads), 0, st, a.src, a.n, Y, a.npad, a.pad2orig, a.nrhs, mk, b);
   ++a.launches;
   // gather: persistent, one block per SM; a stage buffer holds a dense 64-row tile half and <= 8
   // source rows (padded by 16 bytes), as many stages as fit (<= GMAXSTG)
@@ -1560,7 +1603,7 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
       cudaError_t e = launch_chain(lv, false);
       if (e != cudaSuccess) return (int)e;
     }
-    launch_pdl(permute_out_kernel<R>, dim3((unsigned)gblocks), dim3(nthreads), 0, st, Y, a.npad, a.dst, a.n, a.pad2orig, a.nrhs, a.accumulate, mk, b, a.dmax, a.ld_norm);
+    launch_pdl(permute_out_kernel<R>, pgrid, dim3(nthreads), 0, st, Y, a.npad, a.dst, a.n, a.pad2orig, a.nrhs, a.accumulate, mk, b, a.dmax, a.ld_norm);
     ++a.launches;
     return (int)cudaGetLastError();
   }
@@ -1619,7 +1662,7 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
     block_bwd_kernel<R><<<dim3(nb, ny), GT, bsm, st>>>(bs, L, Linv, Y);
     ++a.launches;
   }
-  launch_pdl(permute_out_kernel<R>, dim3((unsigned)gblocks), dim3(nthreads), 0, st, Y, a.npad, a.dst, a.n, a.pad2orig, a.nrhs, a.accumulate, mk, b, a.dmax, a.ld_norm);
+  launch_pdl(permute_out_kernel<R>, pgrid, dim3(nthreads), 0, st, Y, a.npad, a.dst, a.n, a.pad2orig, a.nrhs, a.accumulate, mk, b, a.dmax, a.ld_norm);
   ++a.launches;
   return (int)cudaGetLastError();
 }
@@ -1637,7 +1680,9 @@ int launch_absmax(const double2* V, int64_t n, int nrhs, unsigned* out, cudaStre
 int launch_omega(const unsigned* rmax, const unsigned* xmax, const unsigned* bmax, const unsigned* kmax,
                  const unsigned* dmax, float* dprev, int ninst, int ld, int nrhs, int* done, double tol, double ftol,
                  double* omega, double* stat, cudaStream_t st) {
-  omega_kernel<<<1, 256, 0, st>>>(rmax, xmax, bmax, kmax, dmax, dprev, ninst, ld, nrhs, done, tol, ftol, omega, stat);
+  int width = 1;
+  while (width < nrhs && width < 32) width *= 2;
+  omega_kernel<<<1, 256, 0, st>>>(rmax, xmax, bmax, kmax, dmax, dprev, ninst, ld, nrhs, width, done, tol, ftol, omega, stat);
   return (int)cudaGetLastError();
 }
 
