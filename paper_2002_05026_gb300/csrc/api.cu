@@ -72,8 +72,6 @@ struct d3m_ctx {
   void* E = nullptr;                 // pivot mode: sub-diagonals of the 2 x 2 pivot blocks [NT][b]
   int32_t* piv = nullptr;            // pivot mode: permutation of every diagonal tile [NT][b]
   int64_t* trace = nullptr;
-  TcMaps maps;
-  GatherTcMaps gmaps;                // L's operand planes for the tensor-core solve gathers
   bool gather_tc = false;
   // solve
   SolveItem* fwd_items = nullptr;
@@ -561,20 +559,17 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
     CUDA_TRY(h, cudaMemset(h->E, 0, (size_t)S.NT * b * h->csize));
   }
   if (h->tc) {
-    // operand planes, 8 bytes per complex element either way: bf16 A: [tile][2 splits][2 planes]
-    // [b rows][b], B: [tile][2][2][b][b]; tf32 A and B: [tile][2 planes][b rows][b]
+    // operand planes, 8 bytes per complex element either way, 64-byte swizzled: bf16 A and B
+    // [tile][chunk of 32 columns][2 splits][2 parts][b rows]; tf32 [tile][chunk of 16][2 parts][b rows]
     h->opA = dalloc<unsigned char>(h, (size_t)ntiles * 4 * b * b * 2);
     h->opB = dalloc<unsigned char>(h, (size_t)ntiles * 4 * b * b * 2);
     if (!h->opA || !h->opB) return set_err(h, D3M_ERR_OOM, "cudaMalloc failed for the tensor-core operands");
-    std::string e2;
-    if (tc_make_maps(h->opA, h->opB, ntiles, h->tf32, &h->maps, e2) != 0) return set_err(h, D3M_ERR_CUDA, e2);
     // the solve's off-block products run on the tensor cores from bf16 split planes of L: the
     // BF16x3 engine's own opA, or (TF32) a copy in that layout written beside the tf32 planes
     if (h->tf32) {
       h->opS = dalloc<unsigned char>(h, (size_t)ntiles * 4 * b * b * 2);
       if (!h->opS) return set_err(h, D3M_ERR_OOM, "cudaMalloc failed for the solve operand planes");
     }
-    if (gather_tc_make_maps(h->tf32 ? h->opS : h->opA, ntiles, &h->gmaps, e2) != 0) return set_err(h, D3M_ERR_CUDA, e2);
     h->gather_tc = true;
   }
   // solve
@@ -979,7 +974,7 @@ static int enqueue_factor(d3m_ctx* h, const void* Kin, bool kdev, cudaStream_t s
   p.piv = h->piv;
   if (h->trace) CUDA_TRY(h, cudaMemsetAsync(h->trace, 0xff, (size_t)10 * ntiles * sizeof(int64_t), st));
   ev_begin(h, d3m_ctx::EV_FACTOR, st);
-  if (h->tc) rc = launch_factor_tc(p, h->maps, h->tf32, h->nsm, st);
+  if (h->tc) rc = launch_factor_tc(p, h->tf32, h->nsm, st);
   else if (h->dig) rc = launch_factor_dig(p, h->nsm, st);
   else rc = launch_factor_simt(p, h->fp64, h->nsm, st);
   if (rc) return set_err(h, D3M_ERR_CUDA, std::string("factor launch: ") + cudaGetErrorString((cudaError_t)rc));
@@ -1080,7 +1075,7 @@ static int sweep(d3m_ctx* h, const double2* src, double2* dst, int nrhs, int acc
   a.tinst = h->tinst;
   a.dmax = h->dmax;
   a.ld_norm = h->opt.max_nrhs;
-  a.tcmaps = h->gather_tc ? &h->gmaps : nullptr;
+  a.planes = h->gather_tc ? (h->tf32 ? h->opS : h->opA) : nullptr;
   a.E = h->E;
   a.nsm = h->nsm;
   ev_begin(h, d3m_ctx::EV_SWEEP, st);

@@ -17,11 +17,12 @@
 // bit) to the real half and A_i B_r^T to the imaginary half: [Re | Im] of A B^T.
 //
 // Data movement: every finished L tile is written once, by its owner, as operand planes
-// (opA: L_IJ; opB: W_IJ = L_IJ D_J, or T_J = D_J^{-1} L_JJ^{-1} for a diagonal tile), row-major
-// with the K index contiguous: bf16 [hi_r, hi_i, lo_r, lo_i] / [hi, lo] x [W_r, W_i] (512 rows of
-// 256 bytes), or tf32 [r, i] (256 rows of 512 bytes), 128 KB per tile either way; the TF32
-// engine also writes bf16 split planes of every off-diagonal L tile (opS) for the solve.  TMA
-// tiled loads (64-byte swizzle) stage K chunks of 64-byte rows (32 bf16 or 16 tf32 elements) into
+// (opA: L_IJ; opB: W_IJ = L_IJ D_J, or T_J = D_J^{-1} L_JJ^{-1} for a diagonal tile): for every chunk
+// of 64 bytes of K (32 bf16 or 16 tf32 elements), planes of 128 rows, bf16 [hi_r, hi_i, lo_r, lo_i] or
+// tf32 [r, i], swizzled as the MMA reads them; 128 KB per tile either way.  The TF32
+// engine also writes bf16 split planes of every off-diagonal L tile (opS) for the solve.  A stage is one
+// bulk copy of contiguous bytes per operand (tensor-map boxes of 64-byte rows: 8 x 8 m = 512 12.5 ms where this
+// takes 12.1, one 2 x 2 system of 64 0.20 -> 0.19) into
 // shared memory for the MMAs.  A paired update task (TF32 engine) stages one A chunk with the B
 // chunks of two tiles (I, J) and (I, J + 1) and accumulates them in TMEM columns 0-255 and 256-511.
 //
@@ -35,11 +36,8 @@
 // task share one loop that forms S and the K entries take one address each (142 KB), and a diagonal tile
 // skips its panels of padding.  Diagonal task 92 -> 69 us (m = 512), 82 -> 39 us (m = 64); factorizations: 3 x 3 x 3
 // grid of uneven blocks 5.7 -> 4.3 ms, 4 x 4 m = 512 4.3 -> 3.6, 8 x 8 m = 256 5.3 -> 4.4, 8 x 8 m = 512 13.4 -> 12.5.
-#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
-
-#include <cstring>
 
 #include "device.cuh"
 #include "kernels.h"
@@ -59,19 +57,18 @@ template <> struct Eng<false> {                 // split-BF16x3
   static constexpr int NPA = 4, NPB = 4;        // planes per stage: A [hi_r, hi_i, lo_r, lo_i], B [hi, lo] x [r, i]
   static constexpr int NB = 1;                  // B operands per stage (no paired update tasks)
   static constexpr int NSTAGE = 3;              // GEMM pipeline depth (3 x 64 KB)
-  static constexpr uint32_t ROWS = 512;         // operand rows of one tile in global memory
 };
 template <> struct Eng<true> {                  // TF32
   static constexpr int KC = 16;
   static constexpr int NPA = 2, NPB = 2;        // A [r, i], B [r, i]
   static constexpr int NB = 2;                  // B operands per stage: a paired task's two tiles
   static constexpr int NSTAGE = 4;              // 4 x 48 KB
-  static constexpr uint32_t ROWS = 256;
 };
 template <bool TF> constexpr uint32_t stage_a() { return Eng<TF>::NPA * PLANE; }
 template <bool TF> constexpr uint32_t stage_b() { return Eng<TF>::NPB * PLANE; }
 template <bool TF> constexpr uint32_t stage_ab() { return stage_a<TF>() + stage_b<TF>(); }
 template <bool TF> constexpr uint32_t stage_slot() { return stage_a<TF>() + Eng<TF>::NB * stage_b<TF>(); }
+constexpr int64_t OPTILE = 128 * 1024;          // bytes of one tile's operand planes in global memory
 constexpr uint32_t SMEM_S = 0;                  // TRSM A operand: TB / KC chunks of stage_a (128 KB)
 constexpr uint32_t SMEM_T = 128 * 1024;         // TRSM B stages (2 x stage_b)
 constexpr uint32_t SMEM_BYTES = 192 * 1024;
@@ -120,17 +117,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
 }
 
 // ------------------------------------------------------------------ TMA
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
+// `bytes` contiguous bytes (16-byte aligned, a multiple of 16) into shared memory
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+               "r"(bytes), "r"(bar)
+               : "memory");
 }
 __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
 }
 
 // ------------------------------------------------------------------ tcgen05
@@ -207,6 +201,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Operand planes of a tile in global memory: for every chunk (64 bytes of each row) its NP planes of 128 rows,
+// stored 64-byte swizzled as the MMA reads them, so that a stage is one contiguous bulk copy per operand.
+// Index, in 16-byte units, of unit u of row r of a plane:
+template <int NP>
+__device__ __forceinline__ int op_unit(int plane, int r, int u) {
+  return ((((u >> 2) * NP + plane) * TB + r) << 2) + ((u & 3) ^ ((r >> 1) & 3));
 }
 
 // ------------------------------------------------------------------ bf16 split helpers
@@ -556,12 +558,10 @@ __device__ __forceinline__ void diag_panel_update(float2* sS, const float2* Wt, 
 
 template <bool TF>
 __global__ void __launch_bounds__(NTHR, 1)
-    factor_tc_kernel(const FactorParams p, const __grid_constant__ CUtensorMap mapA,
-                     const __grid_constant__ CUtensorMap mapB) {
+    factor_tc_kernel(const FactorParams p) {
   constexpr int KC = Eng<TF>::KC, NSTAGE = Eng<TF>::NSTAGE, NCH = TB / KC;
   constexpr uint32_t STAGE_A = stage_a<TF>(), STAGE_B = stage_b<TF>(), STAGE = stage_ab<TF>();
   constexpr uint32_t SLOT = stage_slot<TF>();    // bytes between pipeline stages
-  constexpr uint32_t ROWS = Eng<TF>::ROWS;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // 1024-byte alignment of the dynamic region (swizzle atoms); pointer arithmetic on the shared
   // array keeps the accesses in the shared address space
@@ -593,8 +593,6 @@ __global__ void __launch_bounds__(NTHR, 1)
     mbar_init(smem_u32(&bar_acc), 1);
     mbar_init(smem_u32(&bar_acc2), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    tma_prefetch_desc(&mapA);
-    tma_prefetch_desc(&mapB);
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
@@ -659,21 +657,13 @@ __global__ void __launch_bounds__(NTHR, 1)
             const uint32_t s = g_load % NSTAGE, use = g_load / NSTAGE;
             if (!mbar_wait(smem_u32(&bar_empty[s]), (use & 1) ^ 1, deadline)) { failed = true; break; }
             const KEntry ke = p.klist[T.kl_off + c / NCH];
-            const int x = (c % NCH) * KC;
+            const int ch = c % NCH;
             const uint32_t sb = smem_u32(smem + s * SLOT);
             const uint32_t fb = smem_u32(&bar_full[s]);
             mbar_expect_tx(fb, pair ? STAGE + STAGE_B : STAGE);
-#pragma unroll
-            for (int q = 0; q < Eng<TF>::NPA; ++q)
-              tma_load_2d(sb + q * PLANE, &mapA, x, ke.a_tile * (int)ROWS + q * 128, fb);
-#pragma unroll
-            for (int q = 0; q < Eng<TF>::NPB; ++q)
-              tma_load_2d(sb + STAGE_A + q * PLANE, &mapB, x, ke.b_tile * (int)ROWS + q * 128, fb);
-            if (pair) {
-#pragma unroll
-              for (int q = 0; q < Eng<TF>::NPB; ++q)
-                tma_load_2d(sb + STAGE + q * PLANE, &mapB, x, ke.b2_tile * (int)ROWS + q * 128, fb);
-            }
+            bulk_load(sb, opA + ke.a_tile * OPTILE + ch * STAGE_A, STAGE_A, fb);
+            bulk_load(sb + STAGE_A, opB + ke.b_tile * OPTILE + ch * STAGE_B, STAGE_B, fb);
+            if (pair) bulk_load(sb + STAGE, opB + ke.b2_tile * OPTILE + ch * STAGE_B, STAGE_B, fb);
             ++g_load;
           }
         }
@@ -720,9 +710,7 @@ __global__ void __launch_bounds__(NTHR, 1)
         const uint32_t sb = smem_u32(smem + SMEM_T + s * STAGE_B);
         const uint32_t fb = smem_u32(&bar_tfull[s]);
         mbar_expect_tx(fb, STAGE_B);
-#pragma unroll
-        for (int q = 0; q < Eng<TF>::NPB; ++q)
-          tma_load_2d(sb + q * PLANE, &mapB, c * KC, T.diag * (int)ROWS + q * 128, fb);
+        bulk_load(sb, opB + T.diag * OPTILE + c * STAGE_B, STAGE_B, fb);
         ++t_load;
       }
     }
@@ -842,7 +830,7 @@ __global__ void __launch_bounds__(NTHR, 1)
           // T_J = D^{-1} L^{-1}: row n, columns k (X[n][k] = sS[k][n] for k < n); coalesced 16-byte
           // stores of the planes: bf16 [T_r, T_i] x [hi, lo] (16 threads per 256-byte plane row) or
           // tf32 [T_r, T_i] (32 threads per 512-byte plane row)
-          uint4* Bt = reinterpret_cast<uint4*>(opB + (int64_t)T.tile * ROWS * TB * (TF ? 4 : 2));
+          uint4* Bt = reinterpret_cast<uint4*>(opB + T.tile * OPTILE);
 #pragma unroll 1
           for (int it = warp; it < TB * 16 / 32; it += NTHR / 32) {
             // a warp takes 8 rows n by 4 groups of 8 columns: loads of sS[k][n] two to a bank, stores of
@@ -859,10 +847,10 @@ __global__ void __launch_bounds__(NTHR, 1)
               ti[k8] = tv.y;
             }
             if constexpr (TF) {
-              Bt[(0 * 128 + n) * 32 + 2 * c8] = pack4_tf32(tr);
-              Bt[(0 * 128 + n) * 32 + 2 * c8 + 1] = pack4_tf32(tr + 4);
-              Bt[(1 * 128 + n) * 32 + 2 * c8] = pack4_tf32(ti);
-              Bt[(1 * 128 + n) * 32 + 2 * c8 + 1] = pack4_tf32(ti + 4);
+              Bt[op_unit<2>(0, n, 2 * c8)] = pack4_tf32(tr);
+              Bt[op_unit<2>(0, n, 2 * c8 + 1)] = pack4_tf32(tr + 4);
+              Bt[op_unit<2>(1, n, 2 * c8)] = pack4_tf32(ti);
+              Bt[op_unit<2>(1, n, 2 * c8 + 1)] = pack4_tf32(ti + 4);
             } else {
               __nv_bfloat16 h[2][8], lo[2][8];
 #pragma unroll
@@ -872,8 +860,8 @@ __global__ void __launch_bounds__(NTHR, 1)
               }
 #pragma unroll
               for (int pl = 0; pl < 2; ++pl) {
-                Bt[((0 * 256 + pl * 128) + n) * 16 + c8] = pack8(h[pl]);
-                Bt[((1 * 256 + pl * 128) + n) * 16 + c8] = pack8(lo[pl]);
+                Bt[op_unit<4>(pl, n, c8)] = pack8(h[pl]);
+                Bt[op_unit<4>(2 + pl, n, c8)] = pack8(lo[pl]);
               }
             }
           }
@@ -894,9 +882,7 @@ __global__ void __launch_bounds__(NTHR, 1)
               const uint32_t sb = smem_u32(smem + SMEM_T + s * STAGE_B);
               const uint32_t fb = smem_u32(&bar_tfull[s]);
               mbar_expect_tx(fb, STAGE_B);
-#pragma unroll
-              for (int q = 0; q < Eng<TF>::NPB; ++q)
-                tma_load_2d(sb + q * PLANE, &mapB, c * KC, T.diag * (int)ROWS + q * 128, fb);
+              bulk_load(sb, opB + T.diag * OPTILE + c * STAGE_B, STAGE_B, fb);
               ++t_load;
             }
           }
@@ -948,11 +934,12 @@ __global__ void __launch_bounds__(NTHR, 1)
         // ---------------------------------------------------------------- phase 4: store L_IJ
         // operand planes opA (L) and opB (W = L D_J), 16 bytes per thread; the complex64 copy of L
         // (read only by the solve sweeps) is written after the release, below
-        uint4* A = reinterpret_cast<uint4*>(opA + (int64_t)T.tile * ROWS * TB * (TF ? 4 : 2));
-        uint4* B = reinterpret_cast<uint4*>(opB + (int64_t)T.tile * ROWS * TB * (TF ? 4 : 2));
+        uint4* A = reinterpret_cast<uint4*>(opA + T.tile * OPTILE);
+        uint4* B = reinterpret_cast<uint4*>(opB + T.tile * OPTILE);
 #pragma unroll 1
-        for (int it = tid; it < TB * 16; it += NTHR) {
-          const int rr = it >> 4, c8 = it & 15;   // row, group of 8 columns
+        for (int it = warp; it < TB * 16 / 32; it += NTHR / 32) {
+          // row, group of 8 columns: a warp takes 8 rows by 4 groups, 512 contiguous bytes of a plane
+          const int rr = (it >> 2) * 8 + (lane >> 2), c8 = (it & 3) * 4 + (lane & 3);
           float2 l[8];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
@@ -971,27 +958,28 @@ __global__ void __launch_bounds__(NTHR, 1)
             pv[3][k] = w.y;
           }
           if constexpr (TF) {
-            // opA rows: plane * 128 + row (L_r, L_i); opB rows: the same for W; 32 uint4 per 512-byte row
+            // planes L_r, L_i and W_r, W_i
 #pragma unroll
             for (int pl = 0; pl < 2; ++pl) {
-              A[(pl * 128 + rr) * 32 + 2 * c8] = pack4_tf32(pv[pl]);
-              A[(pl * 128 + rr) * 32 + 2 * c8 + 1] = pack4_tf32(pv[pl] + 4);
-              B[(pl * 128 + rr) * 32 + 2 * c8] = pack4_tf32(pv[2 + pl]);
-              B[(pl * 128 + rr) * 32 + 2 * c8 + 1] = pack4_tf32(pv[2 + pl] + 4);
+              A[op_unit<2>(pl, rr, 2 * c8)] = pack4_tf32(pv[pl]);
+              A[op_unit<2>(pl, rr, 2 * c8 + 1)] = pack4_tf32(pv[pl] + 4);
+              B[op_unit<2>(pl, rr, 2 * c8)] = pack4_tf32(pv[2 + pl]);
+              B[op_unit<2>(pl, rr, 2 * c8 + 1)] = pack4_tf32(pv[2 + pl] + 4);
             }
             if (p.opS) {
               // bf16 split planes of L for the solve's tensor-core products, in the layout of the
-              // split-BF16x3 engine's opA (rows split * 256 + plane * 128 + row)
+              // split-BF16x3 engine's opA
               __nv_bfloat16 h[2][8], lo[2][8];
 #pragma unroll
               for (int q = 0; q < 2; ++q)
 #pragma unroll
                 for (int k = 0; k < 8; ++k) split2(pv[q][k], h[q][k], lo[q][k]);
-              uint4* Sp = reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(p.opS) + (int64_t)T.tile * 512 * TB * 2);
-              Sp[((0 * 256 + 0 * 128) + rr) * 16 + c8] = pack8(h[0]);
-              Sp[((0 * 256 + 1 * 128) + rr) * 16 + c8] = pack8(h[1]);
-              Sp[((1 * 256 + 0 * 128) + rr) * 16 + c8] = pack8(lo[0]);
-              Sp[((1 * 256 + 1 * 128) + rr) * 16 + c8] = pack8(lo[1]);
+              uint4* Sp = reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(p.opS) + T.tile * OPTILE);
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                Sp[op_unit<4>(q, rr, c8)] = pack8(h[q]);
+                Sp[op_unit<4>(2 + q, rr, c8)] = pack8(lo[q]);
+              }
             }
           } else {
             __nv_bfloat16 h[4][8], lo[4][8];
@@ -999,16 +987,13 @@ __global__ void __launch_bounds__(NTHR, 1)
             for (int q = 0; q < 4; ++q)
 #pragma unroll
               for (int k = 0; k < 8; ++k) split2(pv[q][k], h[q][k], lo[q][k]);
-            // opA rows: split * 256 + plane * 128 + row; 16 uint4 per 256-byte row
-            A[((0 * 256 + 0 * 128) + rr) * 16 + c8] = pack8(h[0]);
-            A[((0 * 256 + 1 * 128) + rr) * 16 + c8] = pack8(h[1]);
-            A[((1 * 256 + 0 * 128) + rr) * 16 + c8] = pack8(lo[0]);
-            A[((1 * 256 + 1 * 128) + rr) * 16 + c8] = pack8(lo[1]);
-            // opB rows: split * 256 + plane * 128 + row (planes W_r, W_i)
+            // planes hi_r, hi_i, lo_r, lo_i of L and of W
 #pragma unroll
             for (int pl = 0; pl < 2; ++pl) {
-              B[((0 * 256 + pl * 128) + rr) * 16 + c8] = pack8(h[2 + pl]);
-              B[((1 * 256 + pl * 128) + rr) * 16 + c8] = pack8(lo[2 + pl]);
+              A[op_unit<4>(pl, rr, c8)] = pack8(h[pl]);
+              A[op_unit<4>(2 + pl, rr, c8)] = pack8(lo[pl]);
+              B[op_unit<4>(pl, rr, c8)] = pack8(h[2 + pl]);
+              B[op_unit<4>(2 + pl, rr, c8)] = pack8(lo[2 + pl]);
             }
           }
         }
@@ -1062,56 +1047,12 @@ __global__ void __launch_bounds__(NTHR, 1)
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
-// ------------------------------------------------------------------ host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-int tc_make_maps(void* opA, void* opB, int64_t ntiles, bool tf32, TcMaps* out, std::string& err) {
-  static EncodeTiledFn encode = nullptr;
-  if (!encode) {
-    cudaDriverEntryPointQueryResult q;
-    void* fn = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess || !fn) {
-      cudaGetLastError();
-      err = "cuTensorMapEncodeTiled is not available from the driver";
-      return 1;
-    }
-    encode = (EncodeTiledFn)fn;
-  }
-  static_assert(sizeof(CUtensorMap) == 128, "CUtensorMap size");
-  // rows of 128 elements (256 bytes bf16, 512 bytes tf32); a box is one chunk (64 bytes) of 128 rows
-  const int esz = tf32 ? 4 : 2;
-  const cuuint64_t rows = (cuuint64_t)(tf32 ? Eng<true>::ROWS : Eng<false>::ROWS);
-  const cuuint32_t box[2] = {(cuuint32_t)(64 / esz), (cuuint32_t)TB};
-  const cuuint32_t estr[2] = {1, 1};
-  const cuuint64_t stride[1] = {(cuuint64_t)TB * esz};
-  const CUtensorMapDataType dt = tf32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-  CUtensorMap ma, mb;
-  const cuuint64_t dim[2] = {(cuuint64_t)TB, (cuuint64_t)ntiles * rows};
-  CUresult r1 = encode(&ma, dt, 2, opA, dim, stride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
-                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  CUresult r2 = encode(&mb, dt, 2, opB, dim, stride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
-                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r1 != CUDA_SUCCESS || r2 != CUDA_SUCCESS) {
-    err = "cuTensorMapEncodeTiled failed (" + std::to_string((int)r1) + ", " + std::to_string((int)r2) + ")";
-    return 1;
-  }
-  std::memcpy(out->a, &ma, 128);
-  std::memcpy(out->b, &mb, 128);
-  return 0;
-}
-
-int launch_factor_tc(const FactorParams& p, const TcMaps& maps, bool tf32, int nblocks, cudaStream_t st) {
+int launch_factor_tc(const FactorParams& p, bool tf32, int nblocks, cudaStream_t st) {
   const size_t smem = SMEM_BYTES + 1024;   // + alignment slack
   auto kern = tf32 ? factor_tc_kernel<true> : factor_tc_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
-  CUtensorMap ma, mb;
-  std::memcpy(&ma, maps.a, 128);
-  std::memcpy(&mb, maps.b, 128);
-  kern<<<nblocks, NTHR, smem, st>>>(p, ma, mb);
+  kern<<<nblocks, NTHR, smem, st>>>(p);
   return (int)cudaGetLastError();
 }
 

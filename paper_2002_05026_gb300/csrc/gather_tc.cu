@@ -10,9 +10,10 @@
 //
 // Arithmetic: split-BF16x3 products (a = hi + lo; hi*hi + hi*lo + lo*hi) accumulated in FP32 in
 // tensor memory, the same operands and accuracy as the factorization's tile engine.  The L tiles
-// are read from the bf16 operand planes that the factorization wrote (hi_r, hi_i, lo_r, lo_i; row
-// major, 128 x 128), K-major for the forward product and, for the backward product L^T, through
-// the MMA's transposed-A (MN-major) mode with 32 x 32 boxes of the same planes.  The source
+// are read from the bf16 operand planes that the factorization wrote (chunks of 32 columns, in each the planes
+// hi_r, hi_i, lo_r, lo_i of 128 rows, swizzled) by bulk copies, K-major for the forward product (a chunk is one copy)
+// and, for the backward product L^T, through the MMA's transposed-A (MN-major) mode (32 rows of every plane and
+// chunk, 2 KB each).  The source
 // vectors are split to bf16 hi/lo in shared memory by four builder warps: for a chunk of 32 source
 // rows, B planes of N = 2 NR rows [Re | Im outputs] for the real part ([y_r; y_i]) and the
 // imaginary part ([-y_i; y_r]) of A, so every MMA (M = 128, N = 2 NR) adds both parts of the
@@ -22,12 +23,8 @@
 // write the partials (TMEM lanes 32 (w % 4) ..), warps 6..9 build the source planes.  Four
 // 48 KB stages (one 32-row chunk of one item), two TMEM accumulators (the epilogue of one unit
 // overlaps the next unit's products).
-#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
-
-#include <cstring>
-#include <string>
 
 #include "d3m.h"
 #include "device.cuh"
@@ -71,11 +68,10 @@ __device__ __forceinline__ bool gbar_wait(uint32_t bar, uint32_t parity, uint64_
     if (globaltimer_ns() > deadline) return false;
   }
 }
-__device__ __forceinline__ void gtma_2d(uint32_t dst, const void* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
+__device__ __forceinline__ void gbulk(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+               "r"(bytes), "r"(bar)
+               : "memory");
 }
 // 64-byte swizzle descriptors.  K-major: 8-row groups 512 bytes apart (leading offset unused).
 // MN-major (backward A = L^T): 32-element MN groups lbo bytes apart, 8-row K groups 512 apart.
@@ -126,8 +122,7 @@ __device__ __forceinline__ void gsplit(float a, unsigned short& hi, unsigned sho
 template <bool FWD>
 __global__ void __launch_bounds__(GTH, 1)
     gather_tc_kernel(const SolveGroup* __restrict__ groups, const SolveItem* __restrict__ items,
-                     const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapT,
-                     const float2* __restrict__ Y, float2* __restrict__ P, int64_t npad, int nrhs, int NR,
+                     const unsigned char* __restrict__ planes, const float2* __restrict__ Y, float2* __restrict__ P, int64_t npad, int nrhs, int NR,
                      int* status, const int* __restrict__ done, const int32_t* __restrict__ tinst, int nunits) {
   extern __shared__ __align__(1024) unsigned char gsm_raw[];
   unsigned char* smem = gsm_raw + ((1024u - (su32g(gsm_raw) & 1023u)) & 1023u);
@@ -181,23 +176,20 @@ __global__ void __launch_bounds__(GTH, 1)
         if (masked(u)) continue;
         const SolveGroup g = groups[u];
         for (int q = 0; q < g.count && ok; ++q) {
-          const int64_t row0 = (int64_t)items[g.first + q].tile * 512;   // opA rows of the tile
+          const unsigned char* src = planes + items[g.first + q].tile * (int64_t)(4 * GA_STAGE);
           for (int c = 0; c < 4; ++c, ++it) {
             const uint32_t s = it % GNST, use = it / GNST;
             if (!gbar_wait(su32g(&s_empty[s]), (use & 1) ^ 1, deadline)) { ok = false; break; }
             const uint32_t fb = su32g(&a_full[s]);
             gbar_expect_tx(fb, GA_STAGE);
             const uint32_t sa = su32g(smem + s * GSTG);
+            if (FWD) {
+              gbulk(sa, src + c * GA_STAGE, GA_STAGE, fb);                    // columns 32 c .. of all rows
+            } else {
 #pragma unroll
-            for (int pl = 0; pl < 4; ++pl) {
-              // planes hi_r, hi_i, lo_r, lo_i at opA rows split * 256 + part * 128 (pl = 2 split + part)
-              const int prow = (int)(row0 + (pl >> 1) * 256 + (pl & 1) * 128);
-              if (FWD) {
-                gtma_2d(sa + pl * GPLANE, &mapK, c * 32, prow, fb);          // rows r, columns c0..c0+31
-              } else {
-#pragma unroll
-                for (int mc = 0; mc < 4; ++mc)                                // rows c0..c0+31, all columns
-                  gtma_2d(sa + pl * GPLANE + mc * 2048, &mapT, mc * 32, prow + c * 32, fb);
+              for (int q4 = 0; q4 < 16; ++q4) {                               // rows 32 c .., column chunk mc
+                const int pl = q4 >> 2, mc = q4 & 3;
+                gbulk(sa + pl * GPLANE + mc * 2048, src + mc * GA_STAGE + pl * GPLANE + c * 2048, 2048, fb);
               }
             }
           }
@@ -369,52 +361,13 @@ __global__ void __launch_bounds__(GTH, 1)
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128u) : "memory");
 }
 
-// Tensor maps of the operand planes of L for the solve: box {32, 128} (forward, K-major) and
-// {32, 32} (backward, read as MN-major blocks), both with the 64-byte swizzle.
-int gather_tc_make_maps(void* opA, int64_t ntiles, GatherTcMaps* out, std::string& err) {
-  typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                               const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                               CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static EncodeFn encode = nullptr;
-  if (!encode) {
-    cudaDriverEntryPointQueryResult q;
-    void* fn = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess || !fn) {
-      cudaGetLastError();
-      err = "cuTensorMapEncodeTiled is not available from the driver";
-      return 1;
-    }
-    encode = (EncodeFn)fn;
-  }
-  const cuuint64_t dim[2] = {128, (cuuint64_t)ntiles * 512};
-  const cuuint64_t stride[1] = {256};
-  const cuuint32_t estr[2] = {1, 1};
-  for (int k = 0; k < 2; ++k) {
-    const cuuint32_t box[2] = {32, k == 0 ? 128u : 32u};
-    CUtensorMap m;
-    const CUresult r = encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, opA, dim, stride, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-      err = "cuTensorMapEncodeTiled (solve operands) failed: " + std::to_string((int)r);
-      return 1;
-    }
-    std::memcpy(k == 0 ? out->k : out->t, &m, 128);
-  }
-  return 0;
-}
-
-int launch_gather_tc(bool fwd, const GatherTcMaps& maps, const SolveGroup* groups, const SolveItem* items,
+int launch_gather_tc(bool fwd, const void* planes, const SolveGroup* groups, const SolveItem* items,
                      const void* Y, void* P, int64_t npad, int nrhs, int* status, const int* done,
                      const int32_t* tinst, int nunits, int nsm, cudaStream_t st) {
   const size_t smem = GSMEM + 1024;
   auto kern = fwd ? gather_tc_kernel<true> : gather_tc_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
-  CUtensorMap mk, mt;
-  std::memcpy(&mk, maps.k, 128);
-  std::memcpy(&mt, maps.t, 128);
   // right-hand sides in groups of at most 32 (N = 2 NR <= 64 TMEM columns per accumulator)
   const int ng = (nrhs + 31) / 32;
   const int per = (nrhs + ng - 1) / ng;
@@ -429,7 +382,7 @@ int launch_gather_tc(bool fwd, const GatherTcMaps& maps, const SolveGroup* group
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, kern, groups, items, mk, mt, (const float2*)Y, (float2*)P, npad, nrhs, NR, status, done,
+  e = cudaLaunchKernelEx(&cfg, kern, groups, items, (const unsigned char*)planes, (const float2*)Y, (float2*)P, npad, nrhs, NR, status, done,
                          tinst, nunits);
   return (int)e;
 }

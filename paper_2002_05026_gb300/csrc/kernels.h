@@ -48,20 +48,14 @@ struct SweepLaunch {
   const int64_t* inv_off;          // device [N]: first tile of block k in Inv
   const void* InvT;                // transposed inverse tiles (diagonal included)
   const int64_t* invT_off;         // device [N]: first tile of block k in InvT
-  const struct GatherTcMaps* tcmaps;  // operand-plane maps for the tensor-core gathers, or nullptr
+  const void* planes;              // bf16 operand planes of L for the tensor-core gathers, or nullptr
   const void* E;                   // pivot mode: sub-diagonals of the 2 x 2 blocks of D, or nullptr
   int nsm;
   int64_t launches;                // out: kernels launched by launch_sweep
 };
 
-// Tensor maps of L's bf16 operand planes for the tensor-core gathers of the solve (gather_tc.cu):
-// k = box {32, 128} (forward, K-major), t = box {32, 32} (backward, MN-major blocks).
-struct GatherTcMaps {
-  alignas(64) unsigned char k[128];
-  alignas(64) unsigned char t[128];
-};
-int gather_tc_make_maps(void* opA, int64_t ntiles, GatherTcMaps* out, std::string& err);
-int launch_gather_tc(bool fwd, const GatherTcMaps& maps, const SolveGroup* groups, const SolveItem* items,
+// products of a level on the tensor cores (gather_tc.cu)
+int launch_gather_tc(bool fwd, const void* planes, const SolveGroup* groups, const SolveItem* items,
                      const void* Y, void* P, int64_t npad, int nrhs, int* status, const int* done,
                      const int32_t* tinst, int nunits, int nsm, cudaStream_t st);
 
@@ -109,19 +103,12 @@ int resid_tc_groups(int nrhs, int* NR);
 int launch_resid_tc(const ResidualTc& p, const double2* X, const double2* B, double2* R,
                     int nrhs, int nrtiles, int nblk, int max_rtiles, cudaStream_t st, int64_t* launches);
 
-// Tensor maps (CUtensorMap, 128 bytes each) of the tensor-core operand planes.
-struct TcMaps {
-  alignas(64) unsigned char a[128];
-  alignas(64) unsigned char b[128];
-};
-
 // FP64 (unpivoted) with the tile products as exact digit products on the tensor cores
 constexpr int kDigMaxProducts = 64;    // most tile products of one task
 int launch_factor_dig(const FactorParams& p, int nblocks, cudaStream_t st);
 int launch_factor_simt(const FactorParams& p, bool fp64, int nblocks, cudaStream_t st);
 // tf32 = false: bf16 planes of the split-BF16x3 engine; true: tf32 planes
-int tc_make_maps(void* opA, void* opB, int64_t ntiles, bool tf32, TcMaps* out, std::string& err);
-int launch_factor_tc(const FactorParams& p, const TcMaps& maps, bool tf32, int nblocks, cudaStream_t st);
+int launch_factor_tc(const FactorParams& p, bool tf32, int nblocks, cudaStream_t st);
 int launch_sweep(SweepLaunch& a, bool fp64, cudaStream_t st);
 // Inverses of the unit-lower diagonal blocks (c64 tiles of edge b in {64, 128}), built from L and
 // the inverses of the diagonal tiles: work = (block, tile column) pairs.

@@ -1461,9 +1461,9 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
     if (nsm <= 0) nsm = 1;
   }
   auto launch_gather = [&](bool fwd, int64_t i0, int64_t i1) {
-    if (a.tcmaps && sizeof(R) == 4) {
+    if (a.planes && sizeof(R) == 4) {
       // tensor-core gather (split-BF16x3 on L's operand planes): one unit per group
-      launch_gather_tc(fwd, *a.tcmaps, (fwd ? a.fwd_groups : a.bwd_groups) + i0, fwd ? a.fwd_items : a.bwd_items,
+      launch_gather_tc(fwd, a.planes, (fwd ? a.fwd_groups : a.bwd_groups) + i0, fwd ? a.fwd_items : a.bwd_items,
                        Y, P, a.npad, a.nrhs, a.status, a.done, a.tinst, (int)(i1 - i0), nsm, st);
       return;
     }
@@ -1517,7 +1517,7 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
     cs.mk = mk;
     cs.rrows = (int)rrows;
     // partials per slot of a backward gather
-    const int bsub = a.tcmaps && sizeof(R) == 4 ? 1 : nh;
+    const int bsub = a.planes && sizeof(R) == 4 ? 1 : nh;
     auto launch_chain = [&](int lv, bool fwd) -> cudaError_t {
       const int S = a.lev_maxnt[lv] * nh;
       cs.cl = std::min(CHAIN_MAXCL, S);
@@ -1653,7 +1653,7 @@ static int sweep_impl(SweepLaunch& a, cudaStream_t st) {
       launch_gather(false, i0, i1);
       const int64_t nthr = ntl * b * a.nrhs;
       launch_pdl(reduce_kernel<R>, dim3((unsigned)((nthr + 31) / 32)), dim3(ET), 0, st, a.lev_tiles + a.lev_tile_ptr[lv], (int)ntl,
-                                                                     a.bwd_slot_ptr, P, Y, a.npad, b, a.nrhs, a.tcmaps && sizeof(R) == 4 ? 1 : nh, nullptr, mk);
+                                                                     a.bwd_slot_ptr, P, Y, a.npad, b, a.nrhs, a.planes && sizeof(R) == 4 ? 1 : nh, nullptr, mk);
       a.launches += 2;
     }
     bs.blocks = a.lev_blocks + a.lev_ptr[lv];
