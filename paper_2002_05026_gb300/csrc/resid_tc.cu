@@ -178,7 +178,8 @@ __device__ __forceinline__ int scale_exp(unsigned long long maxbits) {
 }
 
 // ---------------------------------------------------------------- K digits
-// (1) per stored block: max |Re|, |Im| (diagonal entries of a diagonal block excluded) as double
+// (1) per stored block (bound by HBM; a division by the block's height only where the diagonal lies in it, 8 x 8 of
+// 512: 0.35 -> 0.28 ms): max |Re|, |Im| (diagonal entries of a diagonal block excluded) as double
 // bits, and the diagonal entries of the diagonal blocks (applied in FP64 by the residual)
 __global__ void __launch_bounds__(256) kblock_max_kernel(ResidualTc p) {
   const int blk = blockIdx.x;
@@ -187,16 +188,28 @@ __global__ void __launch_bounds__(256) kblock_max_kernel(ResidualTc p) {
   const double2* Kb = p.K + p.kblk_off[blk];
   const int64_t tot = (int64_t)mf * mg;
   unsigned long long mx = 0;
-  for (int64_t i = blockIdx.y * 256 + threadIdx.x; i < tot; i += 256 * gridDim.y) {
-    const double2 v = __ldg(Kb + i);
-    const int c = (int)(i / mf), u = (int)(i - (int64_t)c * mf);
-    if (f == g && u == c) {
-      p.Kdiag[p.xoff_orig[f] + u] = v;
-      continue;
-    }
-    const double a = fmax(fabs(v.x), fabs(v.y));
-    const unsigned long long ab = (unsigned long long)__double_as_longlong(a);
+  const int64_t stride = 256 * gridDim.y;
+  auto take = [&](double2 v) {
+    const unsigned long long ab = (unsigned long long)__double_as_longlong(fmax(fabs(v.x), fabs(v.y)));
     mx = ab > mx ? ab : mx;
+  };
+  if (f != g) {
+    int64_t i = blockIdx.y * 256 + threadIdx.x;
+    for (; i + 3 * stride < tot; i += 4 * stride) {   // four loads in flight
+      double2 v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = __ldg(Kb + i + e * stride);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) take(v[e]);
+    }
+    for (; i < tot; i += stride) take(__ldg(Kb + i));
+  } else {
+    for (int64_t i = blockIdx.y * 256 + threadIdx.x; i < tot; i += stride) {
+      const double2 v = __ldg(Kb + i);
+      const int c = (int)(i / mf), u = (int)(i - (int64_t)c * mf);
+      if (u == c) p.Kdiag[p.xoff_orig[f] + u] = v;
+      else take(v);
+    }
   }
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long t = __shfl_xor_sync(0xffffffffu, mx, o);
@@ -205,15 +218,16 @@ __global__ void __launch_bounds__(256) kblock_max_kernel(ResidualTc p) {
   if ((threadIdx.x & 31) == 0 && mx) atomicMax(p.Kmax_bits + blk, mx);
 }
 
-// (2) digits of the stored blocks: one tile of 128 rows x 32 columns of a stored block K_fg (f >= g) per
-// CTA (101 KB of shared memory: two CTAs per SM).  Every entry's 2 ND digits are extracted once, into
+// (2) digits of the stored blocks: one tile of 64 rows x 32 columns of a stored block K_fg (f >= g) per
+// CTA (50 KB of shared memory: four CTAs per SM, so that the loads, digits and stores of different tiles overlap; 128
+// rows and two CTAs took 1.66 ms for 8 x 8 blocks of 512 where this takes 1.27).  Every entry's 2 ND digits are extracted once, into
 // shared memory (their e4m3 codes, [plane][row u][column c]), and written to the planes of both
 // residual contributions of the block: row block f (untransposed: one 32-column chunk of 128 rows u) and, for
 // f != g, row block g (transposed, by 4 x 4 byte transposes: 32 of the 128 rows c, four 32-column chunks of
 // u).  K is read once, coalesced along u (column-major blocks).  Also adds |K| row sums (rows u) and column
 // sums (rows c of the transposed use) into rowsum, for ||K||_inf.  Bound by HBM: 16 bytes read and 2 x 22
 // written an entry.
-constexpr int KD_U = 128, KD_C = 32, KD_LD = 36;    // tile rows, tile columns, padded bytes of a row
+constexpr int KD_U = 64, KD_C = 32, KD_LD = 36;     // tile rows, tile columns, padded bytes of a row
 constexpr size_t KD_SMEM = (size_t)2 * ND * KD_U * KD_LD;
 
 __global__ void __launch_bounds__(256) kdigits_kernel(ResidualTc p) {
@@ -227,16 +241,16 @@ __global__ void __launch_bounds__(256) kdigits_kernel(ResidualTc p) {
   const int E = scale_exp(p.Kmax_bits[blk]);
   const double2* Kb = p.K + p.kblk_off[blk];
   const bool diag = (f == g);
-  const int tid = threadIdx.x, lane = tid & 31, ul = tid & 127, ch = tid >> 7;
+  const int tid = threadIdx.x, lane = tid & 31, ul = tid % KD_U, ch = tid / KD_U;
   const int u = rt * KD_U + ul;
   if (tid < KD_C) s_cs[tid] = 0.f;
   if (tid < 33) s_code[tid] = e4m3_of(tid - 16);
   __syncthreads();
   float rs = 0.f;
 #pragma unroll 1
-  for (int q = 0; q < KD_C / 8; ++q) {
+  for (int q = 0; q < KD_C * KD_U / 1024; ++q) {
     // four columns c0 .. c0 + 3 of row u
-    const int cl0 = ch * 16 + q * 4;
+    const int cl0 = ch * (KD_C * KD_U / 256) + q * 4;
     double2 v[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -271,11 +285,12 @@ __global__ void __launch_bounds__(256) kdigits_kernel(ResidualTc p) {
   // untransposed planes (row block f): chunk ct, whole 4 KB planes, 16-byte units
   {
     const int nkc = (mg + 31) / 32;
-    unsigned char* base = p.kdig + ((int64_t)p.ks_plane[p.blk_eu[blk]] + ((int64_t)rt * nkc + ct) * 2 * ND) * APLANE;
+    unsigned char* base = p.kdig + ((int64_t)p.ks_plane[p.blk_eu[blk]] + ((int64_t)(rt / 2) * nkc + ct) * 2 * ND) * APLANE;
+    const int r0 = (rt & 1) * KD_U;
     for (int w = tid; w < 2 * ND * KD_U * 2; w += 256) {
-      const int h = w & 1, r = (w >> 1) & 127, pl = w >> 8;
+      const int h = w & 1, r = (w >> 1) % KD_U, pl = w / (2 * KD_U);
       const uint32_t* src = reinterpret_cast<const uint32_t*>(sdig + (pl * KD_U + r) * KD_LD + h * 16);
-      *reinterpret_cast<uint4*>(base + pl * APLANE + swz_unit(r, h)) = make_uint4(src[0], src[1], src[2], src[3]);
+      *reinterpret_cast<uint4*>(base + pl * APLANE + swz_unit(r0 + r, h)) = make_uint4(src[0], src[1], src[2], src[3]);
     }
   }
   // transposed planes (row block g, source f): rows c, 32-column chunks of u; a unit is 16 u x 4 c
@@ -283,9 +298,9 @@ __global__ void __launch_bounds__(256) kdigits_kernel(ResidualTc p) {
     const int nkc = (mf + 31) / 32;
     unsigned char* base = p.kdig + ((int64_t)p.ks_plane[p.blk_et[blk]] + (int64_t)(ct / 4) * nkc * 2 * ND) * APLANE;
     const int r0 = (ct & 3) * KD_C;
-    for (int w = tid; w < 2 * ND * 4 * 16; w += 256) {
-      const int h = w & 1, c4 = (w >> 1) & 7, kcl = (w >> 4) & 3, pl = w >> 6;
-      const int kc = rt * 4 + kcl;
+    for (int w = tid; w < 2 * ND * KD_U / 2; w += 256) {
+      const int h = w & 1, c4 = (w >> 1) & 7, kcl = (w >> 4) % (KD_U / 32), pl = w / (KD_U / 2);
+      const int kc = rt * (KD_U / 32) + kcl;
       if (kc >= nkc) continue;
       const unsigned char* src = sdig + (pl * KD_U + kcl * 32 + h * 16) * KD_LD + c4 * 4;
       uint32_t o[4][4];                              // [c][4 u]
@@ -644,7 +659,7 @@ int launch_kdigits(const ResidualTc& p, int nnzb, int nres, int max_rtiles, int 
   cudaMemsetAsync(p.rowsum, 0, (size_t)p.n * sizeof(float), st);
   kblock_max_kernel<<<dim3((unsigned)nnzb, 8), 256, 0, st>>>(p);
   cudaFuncSetAttribute(kdigits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KD_SMEM);
-  kdigits_kernel<<<dim3((unsigned)nnzb, (unsigned)max_rtiles, (unsigned)(4 * max_rtiles)), 256, KD_SMEM, st>>>(p);
+  kdigits_kernel<<<dim3((unsigned)nnzb, (unsigned)(max_rtiles * (128 / KD_U)), (unsigned)(4 * max_rtiles)), 256, KD_SMEM, st>>>(p);
   rowsum_max_kernel<<<nblk, 128, 0, st>>>(p.rowsum, p.xoff_orig, p.m_orig, p.inst, nblk, p.kmax);
   return (int)cudaGetLastError();
 }
