@@ -31,7 +31,8 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 METRIC = "factor+solve time & TFLOP/s at 1e-9 rel err: mixed-prec vs FP64 block LDLᵀ"
-FP64_PEAK_GFLOPS = 1250.0     # GB300 FP64 nominal (152 SMs x 2.07 GHz x ~4 flop/clk/SM)
+FP64_DIGIT_PAIRS = 34          # bf16 digit products of one FP64-level tile product
+FP64_PEAK_SOURCE = "bf16_tflops/34 (burst; FP64 tile products as 34 exact bf16 digit products)"
 # the residual's products issue on the FP32 pipe in double-float form: 60 FP32 instructions per
 # complex multiply-add (8 flops) and right-hand side
 RESID_PEAK_TFLOPS = 152 * 128 * 2.07e9 * 8 / 60 / 1e12
@@ -358,9 +359,10 @@ def adjoint_arm(args, rank, world, local):
             "kernel_ms": fms, "peak_source": "bf16_tflops/3 (burst)", "traffic": None, "peak_kind": peak_kind}
     if args.precision == "tf32":
         roof.update({"peak": peaks["bf16_tflops"] / 2.0, "peak_source": "bf16_tflops/2 (burst; tf32 dense rate)"})
+    elif args.precision == "fp64":
+        roof.update({"peak": peaks["bf16_tflops"] / FP64_DIGIT_PAIRS, "peak_source": FP64_PEAK_SOURCE})
     elif args.precision != "bf16x3":
-        roof.update({"bound": "alu", "peak": FP64_PEAK_GFLOPS / 1e3 if args.precision == "fp64" else
-                     152 * 2.07e9 * 256 / 1e12, "peak_source": "ALU nominal"})
+        roof.update({"bound": "alu", "peak": 152 * 2.07e9 * 256 / 1e12, "peak_source": "ALU nominal"})
     roof["frac"] = roof["achieved"] / roof["peak"]
     line = {"metric": ADJ_METRIC, "value": 1e3 / ms * world, "unit": "gradients/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True,
@@ -665,7 +667,7 @@ def main():
             pk, unit, bound, pname = peaks["bf16_tflops"] / 2.0, "TFLOP/s", "tensor", \
                 "bf16_tflops/2 (burst; tf32 dense rate = half the bf16 rate, nominal 1.1 vs 2.25 PFLOP/s)"
         elif args.precision == "fp64":
-            pk, unit, bound, pname = FP64_PEAK_GFLOPS / 1e3, "TFLOP/s", "alu", "FP64 nominal 1.25 TFLOP/s"
+            pk, unit, bound, pname = peaks["bf16_tflops"] / FP64_DIGIT_PAIRS, "TFLOP/s", "tensor", FP64_PEAK_SOURCE
         else:
             pk, unit, bound, pname = 152 * 2.07e9 * 256 / 1e12, "TFLOP/s", "alu", "FP32 FMA 152 SMs x 128 x 2 x 2.07 GHz"
         kern.append(("factor_kernel", info["factor_kernel_ms_total"],
@@ -762,10 +764,10 @@ def main():
         fp64 = {"ms_per_step": ms64, "tflops": flops_step / (ms64 * 1e-3) / 1e12,
                 "speedup_mixed_vs_fp64": ms64 / ms, "factor_kernel_ms": fk, "warmup_run": warm64,
                 "steps": args.fp64_steps, "handle_device_bytes": int(i64["device_bytes"]),
-                "factor_roofline": {"bound": "alu", "achieved": i64["factor_flops"] / (fk * 1e-3) / 1e12,
-                                    "peak": FP64_PEAK_GFLOPS / 1e3, "unit": "TFLOP/s",
-                                    "peak_source": "FP64 nominal 1.25 TFLOP/s (not measured)",
-                                    "frac": i64["factor_flops"] / (fk * 1e-3) / 1e12 / (FP64_PEAK_GFLOPS / 1e3)},
+                "factor_roofline": {"bound": "tensor", "achieved": i64["factor_flops"] / (fk * 1e-3) / 1e12,
+                                    "peak": peaks["bf16_tflops"] / FP64_DIGIT_PAIRS, "unit": "TFLOP/s",
+                                    "peak_source": FP64_PEAK_SOURCE,
+                                    "frac": i64["factor_flops"] / (fk * 1e-3) / 1e12 / (peaks["bf16_tflops"] / FP64_DIGIT_PAIRS)},
                 "max_rel_diff_mixed_vs_fp64": rel}
         s64.close()
         del X64
