@@ -32,7 +32,17 @@ if ROOT not in sys.path:
 
 METRIC = "factor+solve time & TFLOP/s at 1e-9 rel err: mixed-prec vs FP64 block LDLᵀ"
 FP64_DIGIT_PAIRS = 34          # bf16 digit products of one FP64-level tile product
-FP64_PEAK_SOURCE = "bf16_tflops/34 (burst; FP64 tile products as 34 exact bf16 digit products)"
+FP64_FMA_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
+
+
+def fp64_peak(info, peaks):
+    """(bound, peak TFLOP/s, its source) of the FP64 factorization with the engine that the handle runs."""
+    if info["fp64_engine"] == 1:
+        return ("tensor", peaks["bf16_tflops"] / FP64_DIGIT_PAIRS,
+                "bf16_tflops/34 (burst; FP64 tile products as 34 exact bf16 digit products)")
+    return "alu", FP64_FMA_TFLOPS, "FP64 FMA 152 SMs x 2 x 2 x 2.07 GHz"
+
+
 # the residual's products issue on the FP32 pipe in double-float form: 60 FP32 instructions per
 # complex multiply-add (8 flops) and right-hand side
 RESID_PEAK_TFLOPS = 152 * 128 * 2.07e9 * 8 / 60 / 1e12
@@ -360,7 +370,7 @@ def adjoint_arm(args, rank, world, local):
     if args.precision == "tf32":
         roof.update({"peak": peaks["bf16_tflops"] / 2.0, "peak_source": "bf16_tflops/2 (burst; tf32 dense rate)"})
     elif args.precision == "fp64":
-        roof.update({"peak": peaks["bf16_tflops"] / FP64_DIGIT_PAIRS, "peak_source": FP64_PEAK_SOURCE})
+        roof.update(dict(zip(("bound", "peak", "peak_source"), fp64_peak(info, peaks))))
     elif args.precision != "bf16x3":
         roof.update({"bound": "alu", "peak": 152 * 2.07e9 * 256 / 1e12, "peak_source": "ALU nominal"})
     roof["frac"] = roof["achieved"] / roof["peak"]
@@ -667,7 +677,8 @@ def main():
             pk, unit, bound, pname = peaks["bf16_tflops"] / 2.0, "TFLOP/s", "tensor", \
                 "bf16_tflops/2 (burst; tf32 dense rate = half the bf16 rate, nominal 1.1 vs 2.25 PFLOP/s)"
         elif args.precision == "fp64":
-            pk, unit, bound, pname = peaks["bf16_tflops"] / FP64_DIGIT_PAIRS, "TFLOP/s", "tensor", FP64_PEAK_SOURCE
+            bound, pk, pname = fp64_peak(info, peaks)
+            unit = "TFLOP/s"
         else:
             pk, unit, bound, pname = 152 * 2.07e9 * 256 / 1e12, "TFLOP/s", "alu", "FP32 FMA 152 SMs x 128 x 2 x 2.07 GHz"
         kern.append(("factor_kernel", info["factor_kernel_ms_total"],
@@ -761,13 +772,13 @@ def main():
         i64 = s64.info()
         rel = (torch.linalg.norm(X_mixed - X64, dim=1) / torch.linalg.norm(X64, dim=1)).max().item()
         fk = i64["factor_kernel_ms_total"] / max(1, i64["factor_kernel_calls"])
+        bound64, peak64, source64 = fp64_peak(i64, peaks)
         fp64 = {"ms_per_step": ms64, "tflops": flops_step / (ms64 * 1e-3) / 1e12,
                 "speedup_mixed_vs_fp64": ms64 / ms, "factor_kernel_ms": fk, "warmup_run": warm64,
                 "steps": args.fp64_steps, "handle_device_bytes": int(i64["device_bytes"]),
-                "factor_roofline": {"bound": "tensor", "achieved": i64["factor_flops"] / (fk * 1e-3) / 1e12,
-                                    "peak": peaks["bf16_tflops"] / FP64_DIGIT_PAIRS, "unit": "TFLOP/s",
-                                    "peak_source": FP64_PEAK_SOURCE,
-                                    "frac": i64["factor_flops"] / (fk * 1e-3) / 1e12 / (peaks["bf16_tflops"] / FP64_DIGIT_PAIRS)},
+                "factor_roofline": {"bound": bound64, "achieved": i64["factor_flops"] / (fk * 1e-3) / 1e12,
+                                    "peak": peak64, "unit": "TFLOP/s", "peak_source": source64,
+                                    "frac": i64["factor_flops"] / (fk * 1e-3) / 1e12 / peak64},
                 "max_rel_diff_mixed_vs_fp64": rel}
         s64.close()
         del X64

@@ -63,8 +63,8 @@ enum {
 /* Arithmetic of the factorization (d3m_options.precision). */
 enum {
   D3M_FP64 = 0,          /* complex128 factors, no refinement; tile products as exact digit products
-                            on tcgen05 tensor cores accumulated in fixed point and rounded once to FP64
-                            (where the device memory is short of them, or a task lists over 64 products: an FP64 SIMT engine) */
+                            on tcgen05 tensor cores accumulated in fixed point and rounded once to FP64,
+                            or by FP64 FMAs (d3m_options.fp64_engine) */
   D3M_MIXED_BF16X3 = 1,  /* complex64 factors; Schur/TRSM products on tcgen05 tensor cores as
                             split-BF16x3 (a = a_hi + a_lo; hi*hi + hi*lo + lo*hi) with FP32
                             accumulation in TMEM; FP64 residual + iterative refinement */
@@ -76,6 +76,14 @@ enum {
                             and (I, J+1) in one task sharing L_IK; the solve's products use bf16
                             split planes of L written beside the tf32 ones; FP64 residual +
                             iterative refinement */
+};
+
+/* Tile products of D3M_FP64 (d3m_options.fp64_engine, d3m_info.fp64_engine). */
+enum {
+  D3M_FP64_AUTO = 0,        /* digits where they can be had, else FMA; d3m_get_info tells which */
+  D3M_FP64_DIGITS = 1,      /* digit products on the tensor cores: 32 bytes of digit words per complex entry
+                               of L beside its 16, and at most 64 tile products a task (see seg_group) */
+  D3M_FP64_FMA = 2          /* FP64 FMAs: no words, about ten times the factorization time */
 };
 
 typedef struct {
@@ -122,6 +130,12 @@ typedef struct {
                                graph are unchanged.  D3M_FP64 and D3M_MIXED_SIMT32 only
                                (D3M_ERR_INVALID otherwise).  0 (default) =
                                unpivoted, scalar D */
+  int32_t fp64_engine;      /* D3M_FP64 only: tile products by D3M_FP64_DIGITS or D3M_FP64_FMA
+                               (create fails where DIGITS cannot be had: D3M_ERR_INVALID if a task lists over 64
+                               products, D3M_ERR_OOM without memory for the words).  D3M_FP64_AUTO (default):
+                               DIGITS if the words fit three quarters of the device memory free at
+                               create, else FMA.  The last bits of a solution differ
+                               between the two */
 } d3m_options;
 
 /* Test hook: upload the task graph with one extra unmet dependency on the last task, so the
@@ -166,7 +180,7 @@ typedef struct {
   double sweep_ms_total;
   int64_t factor_kernel_calls, residual_calls, sweep_calls;
   int32_t instances;        /* independent systems held by the handle (1 unless batched) */
-  int32_t reserved0;
+  int32_t fp64_engine;      /* D3M_FP64_DIGITS or D3M_FP64_FMA; 0 in the mixed modes */
   int64_t prio_tasks;       /* tasks the device scheduler serves first: slack within 8% of the
                                estimated critical path of the task graph */
   /* algorithmic bytes of one FP64 residual r = b - K x: the stored lower blocks of K once in

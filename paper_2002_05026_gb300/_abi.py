@@ -27,6 +27,10 @@ D3M_MIXED_BF16X3 = 1
 D3M_MIXED_SIMT32 = 2
 D3M_MIXED_TF32 = 3
 
+D3M_FP64_AUTO = 0
+D3M_FP64_DIGITS = 1
+D3M_FP64_FMA = 2
+
 D3M_DEBUG_STALL_LAST_TASK = 1
 D3M_DEBUG_TRACE = 2
 
@@ -44,7 +48,7 @@ class d3m_options(ctypes.Structure):
                 ("timeout_ns", c_int64), ("tile", c_int32), ("max_nrhs", c_int32),
                 ("fp64_omega", c_int32), ("debug_flags", c_int32), ("graphs", c_int32), ("seg_group", c_int32),
                 ("prio_slack", c_double), ("refine_fwd_tol", c_double), ("task_cost", c_double * 6),
-                ("pivot", c_int32)]
+                ("pivot", c_int32), ("fp64_engine", c_int32)]
 
 
 class d3m_info(ctypes.Structure):
@@ -59,7 +63,7 @@ class d3m_info(ctypes.Structure):
                 ("kernel_launches", c_int64), ("factor_kernel_ms_total", c_double),
                 ("residual_ms_total", c_double), ("sweep_ms_total", c_double),
                 ("factor_kernel_calls", c_int64), ("residual_calls", c_int64), ("sweep_calls", c_int64),
-                ("instances", c_int32), ("reserved0", c_int32), ("prio_tasks", c_int64),
+                ("instances", c_int32), ("fp64_engine", c_int32), ("prio_tasks", c_int64),
                 ("residual_bytes_fixed", c_double), ("residual_bytes_per_rhs", c_double)]
 
     def as_dict(self) -> dict:

@@ -453,6 +453,10 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
     delete h;
     return set_err(nullptr, D3M_ERR_INVALID, "pivoting needs a SIMT engine (D3M_FP64 or D3M_MIXED_SIMT32)");
   }
+  if (h->fp64 && (h->opt.fp64_engine < D3M_FP64_AUTO || h->opt.fp64_engine > D3M_FP64_FMA)) {
+    delete h;
+    return set_err(nullptr, D3M_ERR_INVALID, "fp64_engine must be D3M_FP64_AUTO, D3M_FP64_DIGITS or D3M_FP64_FMA");
+  }
   std::string err;
   // mixed precision: a tile's Schur updates from up to 8 source blocks form one update task (the
   // per-task epilogue through the accumulator dominates short segments), 32 with TF32 (its
@@ -779,14 +783,19 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
   CUDA_TRY(h, cudaMallocHost(&h->h_stat, 3 * sizeof(double)));
   // FP64: the digit engine, where its words (16 bytes per complex entry of L and of
   // W, beside L itself) leave a quarter of the free memory to the caller; else the SIMT engine,
-  // which needs none of them
-  if (h->fp64) {
+  // which needs none of them.  The caller may ask for one of them, and d3m_get_info tells which one runs.
+  const int want = h->opt.fp64_engine;
+  if (h->fp64 && want != D3M_FP64_FMA) {
     const size_t words = (size_t)ntiles * 2 * b * b * sizeof(unsigned long long), exps = (size_t)ntiles * b;
     size_t mfree = 0, mtotal = 0;
     if (cudaMemGetInfo(&mfree, &mtotal) != cudaSuccess) cudaGetLastError();
     int32_t most = 0;                  // the engine lists a task's products in shared memory
     for (const TileTask& t : S.tasks) most = std::max(most, t.nk);
-    if (most <= kDigMaxProducts && 2 * words <= mfree / 4 * 3) {
+    if (want == D3M_FP64_DIGITS && most > kDigMaxProducts)
+      return set_err(h, D3M_ERR_INVALID, "a task of " + std::to_string(most) + " tile products; the digit engine takes at most " +
+                                             std::to_string(kDigMaxProducts) + " (seg_group)");
+    const bool fits = want == D3M_FP64_DIGITS || 2 * words <= mfree / 4 * 3;
+    if (most <= kDigMaxProducts && fits) {
       h->opA = dalloc<unsigned char>(h, words);
       h->opB = dalloc<unsigned char>(h, words);
       h->expA = dalloc<int32_t>(h, exps);
@@ -803,6 +812,7 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
           }
         h->opA = h->opB = nullptr;
         h->expA = h->expB = nullptr;
+        if (want == D3M_FP64_DIGITS) return set_err(h, D3M_ERR_OOM, "cudaMalloc failed for the digit words");
       }
     }
   }
@@ -1375,6 +1385,7 @@ int d3m_get_info(d3m_handle h, d3m_info* info, void* stream) {
   fill_structure(h->S, info);
   info->device_bytes = h->dev_bytes;
   info->instances = h->ninst;
+  info->fp64_engine = !h->fp64 ? 0 : (h->dig ? D3M_FP64_DIGITS : D3M_FP64_FMA);
   int st = h->last_status;
   {
     int sw = 0;

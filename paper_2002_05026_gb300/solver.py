@@ -16,6 +16,7 @@ from ._abi import check, load
 
 PRECISIONS = {"fp64": _abi.D3M_FP64, "bf16x3": _abi.D3M_MIXED_BF16X3, "simt32": _abi.D3M_MIXED_SIMT32,
               "tf32": _abi.D3M_MIXED_TF32}
+FP64_ENGINES = {"auto": _abi.D3M_FP64_AUTO, "digits": _abi.D3M_FP64_DIGITS, "fma": _abi.D3M_FP64_FMA}
 
 
 def _stream_ptr(stream=None) -> int:
@@ -39,7 +40,7 @@ def _as_colmajor(B):
 
 
 def _options(precision, max_nrhs, refine_tol, refine_max_iter, timeout_ns, fp64_omega, debug_flags, graphs=False,
-             prio_slack=None, seg_group=0, task_cost=None, pivot=False):
+             prio_slack=None, seg_group=0, task_cost=None, pivot=False, fp64_engine="auto"):
     opt = _abi.d3m_default_options()
     opt.precision = PRECISIONS[precision] if isinstance(precision, str) else int(precision)
     opt.max_nrhs = max_nrhs
@@ -57,6 +58,7 @@ def _options(precision, max_nrhs, refine_tol, refine_max_iter, timeout_ns, fp64_
         for q in range(6):
             opt.task_cost[q] = float(task_cost[q])
     opt.pivot = int(bool(pivot))
+    opt.fp64_engine = FP64_ENGINES[fp64_engine] if isinstance(fp64_engine, str) else int(fp64_engine)
     return opt
 
 
@@ -66,13 +68,14 @@ class D3M:
     def __init__(self, colptr, rowidx, m=None, blk_size=None, perm=None, precision="bf16x3",
                  max_nrhs: int = 32, refine_tol: float = 1e-12, refine_max_iter: int = 20,
                  timeout_ns: int = 0, fp64_omega: bool = False, debug_flags: int = 0, graphs: bool = False,
-                 prio_slack=None, seg_group: int = 0, task_cost=None, pivot: bool = False, stream=None):
+                 prio_slack=None, seg_group: int = 0, task_cost=None, pivot: bool = False, stream=None,
+                 fp64_engine="auto"):
         lib = load()
         self._lib = lib
         self.h = c_void_p()
         pat, self._keep = _abi.make_pattern(colptr, rowidx, m, blk_size)
         opt = _options(precision, max_nrhs, refine_tol, refine_max_iter, timeout_ns, fp64_omega, debug_flags, graphs,
-                       prio_slack, seg_group, task_cost, pivot)
+                       prio_slack, seg_group, task_cost, pivot, fp64_engine)
         pp = None
         if perm is not None:
             self._perm = np.ascontiguousarray(perm, dtype=np.int32)
@@ -196,7 +199,7 @@ class D3MBatch(D3M):
 
     def __init__(self, instances, perms=None, precision="bf16x3", max_nrhs: int = 32, refine_tol: float = 1e-12,
                  refine_max_iter: int = 20, timeout_ns: int = 0, fp64_omega: bool = False, debug_flags: int = 0,
-                 graphs: bool = False, task_cost=None, stream=None):
+                 graphs: bool = False, task_cost=None, stream=None, fp64_engine="auto"):
         lib = load()
         self._lib = lib
         self.h = c_void_p()
@@ -220,7 +223,7 @@ class D3MBatch(D3M):
                 ctypes.cast(None, POINTER(c_int32)) if q is None else q.ctypes.data_as(POINTER(c_int32))
                 for q in self._perms])
         opt = _options(precision, max_nrhs, refine_tol, refine_max_iter, timeout_ns, fp64_omega, debug_flags, graphs,
-                       task_cost=task_cost)
+                       task_cost=task_cost, fp64_engine=fp64_engine)
         self.precision = precision
         self.stream = stream
         rc = lib.d3m_create_batch(ctypes.byref(self.h), count, pats, pp, ctypes.byref(opt),
