@@ -134,7 +134,7 @@ typedef struct {
                                (create fails where DIGITS cannot be had: D3M_ERR_INVALID if a task lists over 64
                                products, D3M_ERR_OOM without memory for the words).  D3M_FP64_AUTO (default):
                                DIGITS if the words fit three quarters of the device memory free at
-                               create, else FMA.  The last bits of a solution differ
+                               create (a host K's copy set aside), else FMA.  The last bits of a solution differ
                                between the two */
 } d3m_options;
 

@@ -782,11 +782,13 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
   ALLOC(h->contract, double2, S.N);
   CUDA_TRY(h, cudaMallocHost(&h->h_stat, 3 * sizeof(double)));
   // FP64: the digit engine, where its words (16 bytes per complex entry of L and of
-  // W, beside L itself) leave a quarter of the free memory to the caller; else the SIMT engine,
-  // which needs none of them.  The caller may ask for one of them, and d3m_get_info tells which one runs.
+  // W, beside L itself) leave a quarter of the free memory to the caller and a host K's copy, made by the first
+  // factorization that needs it, still fits; else the SIMT engine, which needs none of them.  The caller may
+  // ask for one of them, and d3m_get_info tells which one runs.
   const int want = h->opt.fp64_engine;
   if (h->fp64 && want != D3M_FP64_FMA) {
     const size_t words = (size_t)ntiles * 2 * b * b * sizeof(unsigned long long), exps = (size_t)ntiles * b;
+    const size_t kcopy = (size_t)S.kblk_off.back() * sizeof(double2);
     size_t mfree = 0, mtotal = 0;
     if (cudaMemGetInfo(&mfree, &mtotal) != cudaSuccess) cudaGetLastError();
     int32_t most = 0;                  // the engine lists a task's products in shared memory
@@ -794,7 +796,7 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
     if (want == D3M_FP64_DIGITS && most > kDigMaxProducts)
       return set_err(h, D3M_ERR_INVALID, "a task of " + std::to_string(most) + " tile products; the digit engine takes at most " +
                                              std::to_string(kDigMaxProducts) + " (seg_group)");
-    const bool fits = want == D3M_FP64_DIGITS || 2 * words <= mfree / 4 * 3;
+    const bool fits = want == D3M_FP64_DIGITS || (mfree > kcopy && 2 * words <= (mfree - kcopy) / 4 * 3);
     if (most <= kDigMaxProducts && fits) {
       h->opA = dalloc<unsigned char>(h, words);
       h->opB = dalloc<unsigned char>(h, words);

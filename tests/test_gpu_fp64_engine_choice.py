@@ -1,7 +1,11 @@
-"""The FP64 tile engine of a handle: which one a handle gets, that it is reported, that either can be asked for, and
-that both give the oracle's solutions on uneven blocks of several tiles."""
+"""The FP64 tile engine of a handle: which one a handle gets, that it is reported, that either can be asked for, that
+both give the oracle's solutions on uneven blocks of several tiles, and that the choice leaves room for the copy of a
+host K."""
 import numpy as np
 import pytest
+
+import oracle as O
+import synth
 
 pytestmark = pytest.mark.gpu
 DIGITS, FMA = 1, 2
@@ -78,3 +82,36 @@ def test_engines_match_the_oracle(torch_cuda, engine, pivot, sizes):
     s.close()
     Xo = np.linalg.solve(K, B)
     assert np.linalg.norm(X - Xo) <= 1e-10 * np.linalg.norm(Xo)      # the bar of the FP64 parity tests
+
+
+def test_room_for_the_copy_of_a_host_k(torch_cuda):
+    # a chain of eight blocks of 1024 without fill: K takes 252 MB, L's tiles 189 and the digit words 378.  With what the
+    # handle needs besides the words, 4/3 of the words and 40 MB free, the words fit three quarters of the rest, but
+    # would leave less than K takes.
+    from paper_2002_05026_gb300 import D3M
+    torch = torch_cuda
+    p = synth.make_problem(9, 1, 1, 1024, 1.0, 0.1, 5)
+    K = p.blocks_numpy()
+    kw = dict(colptr=p.colptr, rowidx=p.rowidx, m=p.m, precision="fp64", max_nrhs=1)
+    B = torch.from_numpy(np.ascontiguousarray(synth.rhs(9, p.n, 1))).cuda()
+    sizes = {}
+    for engine in ("digits", "fma"):                  # both engines' kernels are loaded before memory gets short
+        s = D3M(fp64_engine=engine, **kw)
+        sizes[engine] = s.info()["device_bytes"]
+        s.factor(K)
+        ref = s.solve(B)
+        assert s.info()["status"] == 0
+        s.close()
+    words = sizes["digits"] - sizes["fma"]
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    hog = torch.empty(free - (sizes["fma"] + words * 4 // 3 + (40 << 20)), dtype=torch.uint8, device="cuda")
+    s = D3M(**kw)
+    s.factor(K)                                       # the copy of a host K is allocated here
+    X = s.solve(B)
+    inf = s.info()
+    s.close()
+    del hog
+    torch.cuda.empty_cache()
+    assert inf["status"] == 0 and inf["fp64_engine"] == FMA
+    assert torch.equal(X, ref)                        # ref is the FMA engine's
