@@ -556,11 +556,16 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
       }
       __syncthreads();
       const int nr = T.rv;                          // real unknowns of the tile
-      // max |S| over the real lower triangle (breakdown scale), in FP32 relative to the largest exponent
+      // max |S| over the real lower triangle (breakdown scale), in FP32 relative to the largest exponent; Inf if an
+      // entry is, and a NaN does not count
+      auto mag_exp = [](double2 z) {
+        const int e = max(exp_of(z.x, 0), exp_of(z.y, 0));
+        return e >= X_BAD && (isnan(z.x) || isnan(z.y)) ? X_ZERO : e;
+      };
       int mexp = X_ZERO;
       for (int i = tid; i < TB * TB; i += NTHR) {
         const int r = i >> 6, c = i & 63;
-        if (c <= r && r < nr) mexp = max(mexp, max(exp_of(sS[r * LDS + c].x, 0), exp_of(sS[r * LDS + c].y, 0)));
+        if (c <= r && r < nr) mexp = max(mexp, mag_exp(sS[r * LDS + c]));
       }
       mexp = __reduce_max_sync(0xffffffffu, mexp);
       if (lane == 0) s_mexp[warp] = mexp;
@@ -571,7 +576,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         float mx = 0.f;
         for (int i = tid; i < TB * TB; i += NTHR) {
           const int r = i >> 6, c = i & 63;
-          if (c <= r && r < nr) {
+          if (c <= r && r < nr && mag_exp(sS[r * LDS + c]) != X_ZERO) {
             const float x = to_f32(scale2(sS[r * LDS + c].x, 1023 - mexp)), y = to_f32(scale2(sS[r * LDS + c].y, 1023 - mexp));
             mx = fmaxf(mx, x * x + y * y);
           }
@@ -826,7 +831,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         if (warp == 0) {
           float smx = 0.f;
           for (int w = 0; w < NWK; ++w) smx = fmaxf(smx, s_red[w]);
-          const double smax = scale2((double)sqrtf(smx), mexp - 1023);
+          const double smax = mexp >= X_BAD ? (double)INFINITY : scale2((double)sqrtf(smx), mexp - 1023);
           double amin = 3.0e38, amax = 0.0;
           if constexpr (PIV) {
             bk_pivot_range<double>(s_bk, T.cv, amin, amax);
