@@ -62,9 +62,10 @@ enum {
 
 /* Arithmetic of the factorization (d3m_options.precision). */
 enum {
-  D3M_FP64 = 0,          /* complex128 factors, no refinement; tile products as exact digit products
-                            on tcgen05 tensor cores accumulated in fixed point and rounded once to FP64,
-                            or by FP64 FMAs (d3m_options.fp64_engine) */
+  D3M_FP64 = 0,          /* complex128 factors, no refinement; tile products by FP64 FMAs, or (d3m_options.
+                            fp64_engine) as digit products on tcgen05 tensor cores, accumulated in fixed point
+                            and rounded once to FP64: operands to 2^-55 of their row of a tile's largest entry,
+                            outputs that this would leave short of FP64 by FMAs all the same */
   D3M_MIXED_BF16X3 = 1,  /* complex64 factors; Schur/TRSM products on tcgen05 tensor cores as
                             split-BF16x3 (a = a_hi + a_lo; hi*hi + hi*lo + lo*hi) with FP32
                             accumulation in TMEM; FP64 residual + iterative refinement */

@@ -66,8 +66,8 @@ struct d3m_ctx {
   void* opA = nullptr;
   void* opB = nullptr;
   void* opS = nullptr;               // TF32: bf16 split planes of L for the solve's tensor-core products
-  int32_t* expA = nullptr;           // digit engine: row scales of opA / opB
-  int32_t* expB = nullptr;
+  int4* rowA = nullptr;              // digit engine: row scales of opA / opB and the columns near them
+  int4* rowB = nullptr;
   void* Sacc = nullptr;
   void* E = nullptr;                 // pivot mode: sub-diagonals of the 2 x 2 pivot blocks [NT][b]
   int32_t* piv = nullptr;            // pivot mode: permutation of every diagonal tile [NT][b]
@@ -787,7 +787,7 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
   // ask for one of them, and d3m_get_info tells which one runs.
   const int want = h->opt.fp64_engine;
   if (h->fp64 && want != D3M_FP64_FMA) {
-    const size_t words = (size_t)ntiles * 2 * b * b * sizeof(unsigned long long), exps = (size_t)ntiles * b;
+    const size_t words = (size_t)ntiles * 2 * b * b * sizeof(unsigned long long), rows = (size_t)ntiles * b;
     const size_t kcopy = (size_t)S.kblk_off.back() * sizeof(double2);
     size_t mfree = 0, mtotal = 0;
     if (cudaMemGetInfo(&mfree, &mtotal) != cudaSuccess) cudaGetLastError();
@@ -800,12 +800,12 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
     if (most <= kDigMaxProducts && fits) {
       h->opA = dalloc<unsigned char>(h, words);
       h->opB = dalloc<unsigned char>(h, words);
-      h->expA = dalloc<int32_t>(h, exps);
-      h->expB = dalloc<int32_t>(h, exps);
-      h->dig = h->opA && h->opB && h->expA && h->expB;
+      h->rowA = dalloc<int4>(h, rows);
+      h->rowB = dalloc<int4>(h, rows);
+      h->dig = h->opA && h->opB && h->rowA && h->rowB;
       if (!h->dig) {
-        void* part[4] = {h->opA, h->opB, h->expA, h->expB};
-        const size_t bytes[4] = {words, words, exps * sizeof(int32_t), exps * sizeof(int32_t)};
+        void* part[4] = {h->opA, h->opB, h->rowA, h->rowB};
+        const size_t bytes[4] = {words, words, rows * sizeof(int4), rows * sizeof(int4)};
         for (int q = 0; q < 4; ++q)
           if (part[q]) {
             h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), part[q]));
@@ -813,7 +813,7 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
             cudaFree(part[q]);
           }
         h->opA = h->opB = nullptr;
-        h->expA = h->expB = nullptr;
+        h->rowA = h->rowB = nullptr;
         if (want == D3M_FP64_DIGITS) return set_err(h, D3M_ERR_OOM, "cudaMalloc failed for the digit words");
       }
     }
@@ -974,8 +974,8 @@ static int enqueue_factor(d3m_ctx* h, const void* Kin, bool kdev, cudaStream_t s
   p.opA = h->opA;
   p.opB = h->opB;
   p.opS = h->opS;
-  p.expA = h->expA;
-  p.expB = h->expB;
+  p.rowA = h->rowA;
+  p.rowB = h->rowB;
   p.k_arrived = kup ? h->k_arrived : nullptr;
   p.Sacc = h->Sacc;
   p.trace = h->trace;

@@ -10,8 +10,8 @@
 // Algorithms 2012):
 //  * every row of an operand tile has a scale 2^E above its largest |Re|, |Im| (after a power-of-two
 //    balance of the columns, see balance_of); an entry is held
-//    as the 56-bit integer F = x 2^(54 - E) rounded to nearest (|error| <= 2^-55 of the scale), biased
-//    by 0x80 in each of its seven bytes, so byte s of the word is 128 + the balanced base-256 digit
+//    as the 56-bit integer F = x 2^(54 - E) rounded to nearest (|error| <= 2^-55 of the scale; subnormals as zero),
+//    biased by 0x80 in each of its seven bytes, so byte s of the word is 128 + the balanced base-256 digit
 //    d_s in [-128, 127].  A finished tile is stored in this form beside its complex128 values;
 //  * a digit is an exact bf16.  One tensor-core level t sums the digit products d_s d_q, s + q = t,
 //    over the tile's 64 complex columns (128 terms of the real embedding, at most 7 pairs): an
@@ -20,8 +20,20 @@
 //  * the level sums of a tile product are combined exactly in 64-bit integers and added, aligned
 //    by their scales, to a 128-bit fixed-point sum per output (two 64-bit words) over all products
 //    of the task: a task rounds to FP64 once, at its end.
-// The error of one product, sqrt(128) 2^-54.8 of row maxima, is below that of 128 FP64 FMAs.
-// A row with an Inf or NaN gives NaN outputs.
+// The error of one product is about sqrt(128) 2^-54.8 of the product of the two rows' largest entries, that of FMAs
+// a part 2^-53 of the terms' sum.  So an output of the digits falls short of FP64 where the two rows are large in
+// different columns: unknowns in groups that couple weakly, a coupling that decays, anything but a diagonal scaling,
+// which the balance removes.  Every row therefore carries its near columns, those within 2^-2 of its largest
+// exponent.  Two rows that share one have sum |a_k b_k| >= 2^-6 of the scales' product; an output whose rows share
+// none (or whose scales lie 2^13 below those of the task's largest product, or near the subnormal numbers, or in
+// rows with an Inf or NaN) is formed by FP64 FMAs (fma_outputs).  X_JJ and a panel's X_kk are held without their
+// unit diagonal, whose term is added in FP64: it would set the scale of every row of a dominant tile.  Error of the
+// worst of the groups of unknowns of a dense system, coupled by eps^|g_i - g_j| and driven in one of them (digits
+// alone, digits and FMAs, FMAs alone): two groups, eps = 1e-4: 1.7e-12, 4.8e-16, 7.9e-16; 1e-8: 1.7e-8, 3.5e-16,
+// 6.2e-16; eight groups, eps = 2^-4: 2.4e-8, 1.6e-15, 7e-16; no groups: 4.9e-16, 4.1e-16, 7.1e-16.
+// Cost, 4 x 4 grid, m = 512: dense: 2 % of the tasks have a few such outputs, factorization 20.2 -> 21.4 ms (an update
+// of eight products 104 -> 106 us, an off-diagonal tile 44 -> 51, a diagonal one 162 -> 172); two and eight groups:
+// 250 and 310 ms (FMAs alone: 255).
 //
 // One product: MMA M = 128 rows [Re c | Im c] of the embedded W (rows [b_r | -b_i], then
 // [b_i | b_r]), N up to 448 = digits x 64 rows of L ([a_r | a_i]), K = 16 complex columns a
@@ -33,10 +45,10 @@
 // does not (8 levels x 64 columns fill the tensor memory).
 //
 // Measured on GB300, factorization of a 4 x 4 grid with m = 512 (127 k products): 255 ms with DFMA tile
-// products (1.04 TFLOP/s, 83 % of the FP64 pipe), 20 ms here; 3 x 3 grid with m = 100: 12.3 -> 2.9 ms.  A
+// products (1.04 TFLOP/s, 83 % of the FP64 pipe), 21 ms here; 3 x 3 grid with m = 100: 12.3 -> 3.0 ms.  A
 // product takes about 20 k cycles (DFMA: 524 k), 8.7 k of them MMAs: two stages do not hide the
 // expansion (2 k a stage) behind them, and the read-back (6 k) waits for the last one.  A diagonal tile
-// takes about 120 us, 16 us of it per 16-column pivot chain.  Solutions against 64-bit references: as far off as with DFMA
+// takes about 170 us with the update before it (22 us), 16 us of it per 16-column pivot chain.  Solutions against 64-bit references: as far off as with DFMA
 // (1.4e-15 and 1.1e-15 for these two).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -68,6 +80,7 @@ constexpr int MAXP = kDigMaxProducts;            // products of one task
 constexpr int PW = CH;                           // panel width of a diagonal tile
 constexpr uint32_t SMEM_S = STAGE;               // the tile of a diagonal task, behind one stage
 static_assert(STAGE + TB * LDS * 16 + 2 * TB * (PW + 1) * 8 <= SMEM_BYTES, "shared memory of a diagonal task");
+constexpr uint32_t OLD_OFF = 64 * 1024;          // exponents of S in a triangular solve: short2 [TB][TB]
 constexpr unsigned long long BIAS = 0x0080808080808080ull;
 constexpr int E_BAD = 8192;                      // scale of a row with an Inf or NaN
 static_assert(TB * LDS * 16 <= SMEM_BYTES && STAGE % 1024 == 0, "shared memory");
@@ -135,8 +148,21 @@ __device__ __forceinline__ int exp_of(double x, int shift) {
   const int be = (int)((__double_as_longlong(x) >> 52) & 0x7ff);
   return be == 0 ? X_ZERO : (be == 0x7ff ? X_BAD : be + shift);
 }
-// scale exponent of a row from the largest exp_of its entries
-__device__ __forceinline__ int row_scale(int be) { return be >= X_BAD ? E_BAD : be - 1022; }
+// Row of an operand tile: its scale exponent from the largest exp_of its entries (that of a row of zeros is below
+// every other), and its near columns, within 2^-NEAR of its largest entry (bit k: column k): all for a row of zeros,
+// none with an Inf or NaN, or where a product with it may be subnormal
+constexpr int E_ZERO = -3000, E_TINY = -450;
+constexpr int NEAR = 2;
+__device__ __forceinline__ int row_scale(int be) { return be >= X_BAD ? E_BAD : max(be - 1022, E_ZERO); }
+__device__ __forceinline__ bool near_max(int e, int rowmax) { return e >= rowmax - NEAR; }
+__device__ __forceinline__ bool no_near(int E) { return E >= E_BAD || (E < E_TINY && E > E_ZERO); }
+__device__ __forceinline__ int4 row_info(int rowmax, unsigned lo, unsigned hi) {
+  const int E = row_scale(rowmax);
+  return no_near(E) ? make_int4(E, 0, 0, 0) : make_int4(E, 0, (int)lo, (int)hi);
+}
+constexpr int SLACK = 6;                         // a term beside a product counts if 2^SLACK of it reaches the scales'
+constexpr int SPREAD = 13;                       // bits of the fixed-point sum past a product's own
+constexpr int E_NONE = -100000;
 // biased word of x 2^shift for scale 2^E (|x 2^shift| < 2^E): bytes 6..0 = digits 0..6 plus 128
 __device__ __forceinline__ unsigned long long word_of(double x, int shift, int E) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
@@ -268,6 +294,9 @@ __device__ __forceinline__ double to_f64(float f) {
   const uint32_t u = __float_as_uint(f), e = (u >> 23) & 0xff;
   return e ? __hiloint2double((int)((u & 0x80000000u) | ((((u >> 3) & 0x0fffffffu) + (896u << 20)))), (int)(u << 29)) : 0.0;
 }
+// v + part p of a b, b given as part_of_b(b, p)
+__device__ __forceinline__ double2 part_of_b(double2 b, int p) { return p ? make_double2(b.y, b.x) : make_double2(b.x, -b.y); }
+__device__ __forceinline__ double add_part(double2 a, double2 w, double v) { return fma(a.y, w.y, fma(a.x, w.x, v)); }
 // part p of the complex product u z
 __device__ __forceinline__ double mul_part(double2 u, double2 z, int p) {
   return fma(p ? u.y : -u.y, p ? z.x : z.y, u.x * (p ? z.y : z.x));
@@ -305,6 +334,106 @@ __device__ __forceinline__ double recip_part(double dp, int p) {
   return scale2(t, k);
 }
 
+// Outputs of an update whose digit sum would fall short of FP64 (bit i: output (r0 + i, c)): ex, near: scales and near
+// columns of the n products' rows [n][2 TB]
+__device__ __noinline__ unsigned short_outputs(const short (*ex)[2 * TB], const unsigned long long* near, int n, int r0, int c,
+                                               const int* MA, const int* MB) {
+  unsigned fix = 0;
+#pragma unroll 1
+  for (int i = 0; i < 16; ++i) {
+    int best = E_NONE, rest = E_NONE;              // largest product of scales with a column near both, without
+    for (int e = 0; e < n; ++e) {
+      const int ea = ex[e][r0 + i], eb = ex[e][TB + c];
+      const bool hit = (near[e * 2 * TB + r0 + i] & near[e * 2 * TB + TB + c]) != 0;
+      if (!hit) rest = max(rest, ea + eb);
+      else if (min(ea, eb) > E_ZERO) best = max(best, ea + eb);
+    }
+    if (rest > best || (best > E_NONE && MA[r0 + i] + MB[c] - best > SPREAD)) fix |= 1u << i;
+  }
+  return fix;
+}
+// Outputs by FMAs.  solve: of S and X_JJ without its diagonal, else of the task's n products.
+struct FixArgs {
+  const TileTask* T;
+  const KEntry* kl;
+  const double2 *L, *Linv, *D, *E;                 // E: nullptr without pivoting
+  const int* pm;
+};
+constexpr uint32_t FIX_B = TB * LDS * 16, FIX_LIST = 2 * FIX_B;  // operands [TB][LDS] (then the sums), list
+constexpr int FIX_FEW = 64, FIX_MAX = 10 * NTHR;
+static_assert(FIX_LIST + FIX_MAX * 2 <= SMEM_BYTES, "list of short outputs");
+__device__ __forceinline__ double* fix_sum(unsigned char* smem) { return reinterpret_cast<double*>(smem); }
+__device__ __forceinline__ unsigned short* fix_list(unsigned char* smem) { return reinterpret_cast<unsigned short*>(smem + FIX_LIST); }
+// entries (row, k) of the operands of product e
+__device__ __forceinline__ double2 fix_a(const FixArgs& g, const TileTask& T, bool solve, int e, int r, int k) {
+  const int x = r * TB + k;
+  if (!solve) return ld_cg(g.L + (int64_t)g.kl[T.kl_off + e].a_tile * TB * TB + x);
+  const double* Sa = reinterpret_cast<const double*>(g.L + (int64_t)T.tile * TB * TB);
+  return make_double2(__ldcg(Sa + x), __ldcg(Sa + TB * TB + x));
+}
+__device__ __forceinline__ double2 fix_b(const FixArgs& g, const TileTask& T, bool solve, int e, int r, int k) {
+  const int x = r * TB + k;
+  if (solve) return k == (g.E ? g.pm[r] : r) ? make_double2(0.0, 0.0) : ld_cg(g.Linv + (int64_t)T.col * TB * TB + x);
+  const KEntry ke = g.kl[T.kl_off + e];
+  const double2* b = g.L + (int64_t)ke.b_tile * TB * TB + x;
+  double2 w = cmul(ld_cg(b), ld_cg(g.D + (int64_t)ke.kcol * TB + k));       // W_JK = L_JK D_K
+  if (g.E) {
+    const double2* eK = g.E + (int64_t)ke.kcol * TB + k;
+    if (k + 1 < TB) w = cfma(ld_cg(b + 1), ld_cg(eK), w);
+    if (k > 0) w = cfma(ld_cg(b - 1), ld_cg(eK - 1), w);
+  }
+  return w;
+}
+// the operands of product e in shared memory (all threads)
+__device__ __noinline__ void stage_operands(const FixArgs& g, bool solve, int e, unsigned char* smem) {
+  const TileTask T = *g.T;
+  double2 *fA = reinterpret_cast<double2*>(smem), *fB = reinterpret_cast<double2*>(smem + FIX_B);
+#pragma unroll 4
+  for (int x = threadIdx.x; x < TB * TB; x += NTHR) {
+    fA[(x >> 6) * LDS + (x & 63)] = fix_a(g, T, solve, e, x >> 6, x & 63);
+    fB[(x >> 6) * LDS + (x & 63)] = fix_b(g, T, solve, e, x >> 6, x & 63);
+  }
+  __syncthreads();
+}
+// sums of the `count` <= FIX_MAX outputs of fix_list (part, row, column) into fix_sum (all threads)
+__device__ __noinline__ void fma_outputs(const FixArgs& g, bool solve, int n, unsigned char* smem, int count) {
+  if (count <= FIX_FEW) {                          // a warp an output (staging the tiles takes about 5 us a product)
+    const TileTask T = *g.T;
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int q = threadIdx.x >> 5; q < count; q += NWK) {
+      const int code = fix_list(smem)[q], r = code >> 6 & 63, c = code & 63;
+      double v = 0.0;
+#pragma unroll 2
+      for (int e = 0; e < n; ++e)
+#pragma unroll
+        for (int k = lane; k < TB; k += 32) v = add_part(fix_a(g, T, solve, e, r, k), part_of_b(fix_b(g, T, solve, e, c, k), code >> 12), v);
+      for (int o = 16; o > 0; o >>= 1) v += shfl_d(v, o);
+      if (lane == 0) fix_sum(smem)[q] = v;
+    }
+    __syncthreads();
+    return;
+  }
+  double v[FIX_MAX / NTHR];
+#pragma unroll 1
+  for (int e = 0; e < n; ++e) {
+    stage_operands(g, solve, e, smem);
+#pragma unroll 1
+    for (int q = threadIdx.x, j = 0; q < count; q += NTHR, ++j) {
+      const int code = fix_list(smem)[q];
+      const double2* a = reinterpret_cast<const double2*>(smem) + (code >> 6 & 63) * LDS;
+      const double2* b = reinterpret_cast<const double2*>(smem + FIX_B) + (code & 63) * LDS;
+      double s = e ? v[j] : 0.0;
+#pragma unroll 4
+      for (int k = 0; k < TB; ++k) s = add_part(a[k], part_of_b(b[k], code >> 12), s);
+      v[j] = s;
+    }
+    __syncthreads();
+  }
+  for (int q = threadIdx.x, j = 0; q < count; q += NTHR, ++j) fix_sum(smem)[q] = v[j];
+  __syncthreads();
+}
+
 template <int V> struct IntC { static constexpr int value = V; };
 using I4 = IntC<4>;
 using I16 = IntC<16>;
@@ -323,9 +452,13 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
   __shared__ int s_task, s_pending;
   __shared__ int s_MA[TB], s_MB[TB];              // largest row scales of the task's operands
   __shared__ const unsigned long long *s_fa[MAXP], *s_fb[MAXP];
-  __shared__ const int32_t *s_ea[MAXP], *s_eb[MAXP];
+  __shared__ const int4 *s_ea[MAXP], *s_eb[MAXP];
   __shared__ short s_ex[MAXP][2 * TB];            // row scales of every product of the task
-  __shared__ int s_eL[TB], s_eW[TB];              // scales (biased exponents first) of finished rows
+  __shared__ int s_eL[TB], s_eW[TB];              // largest biased exponents of finished rows
+  __shared__ unsigned s_near[TB][2], s_nearV[TB][2];   // columns near them (L or S, W)
+  __shared__ unsigned short s_nearL[TB], s_nearW[TB];   // the same of a panel product's operands
+  __shared__ int s_pm[TB];                        // pivot mode: the tile's own order
+  __shared__ int s_nfix, s_at;                    // short outputs of a task; listed so far
   __shared__ int s_ek[TB], s_eS[TB];              // balance of every column; the same in the tile's order
   __shared__ BkShared<double2> s_bk;              // pivot mode
   __shared__ double2 s_d[TB], s_dinv[TB], s_u[2][PW], s_x[2][PW], s_dg[2];
@@ -340,8 +473,8 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
   double2* Dg = reinterpret_cast<double2*>(p.D);
   unsigned long long* FL = reinterpret_cast<unsigned long long*>(p.opA);
   unsigned long long* FW = reinterpret_cast<unsigned long long*>(p.opB);
-  int32_t* EL = p.expA;
-  int32_t* EW = p.expB;
+  int4* EL = p.rowA;
+  int4* EW = p.rowB;
   constexpr int64_t TW = 2 * TB * TB;             // words of a tile
 
   if (tid == 0) {
@@ -420,23 +553,75 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
       }
     };
     // products of the n <= MAXP operand pairs listed in s_fa, s_fb (word pointers) and s_ea, s_eb (row
-    // scales): H, Lo = sum of A B^T in units of 2^(MA[r] + MB[c] - 46), - 74
-    auto products = [&](int n) {
+    // scales): H, Lo = sum of A B^T in units of 2^(MA[r] + MB[c] - 46), - 74; the outputs of the mask fix, whose
+    // digits would fall short of FP64, by FMAs: in H as a double.  solve: the one pair is S and X_JJ without its
+    // diagonal; the caller adds S (an output is short only if that term is small too).
+    unsigned fix = 0;
+    auto products = [&](int n, bool solve) {
+      fix = 0;
 #pragma unroll
       for (int i = 0; i < 16; ++i) H[i] = Lo[i] = 0;
+      Words8 w;
+      auto fetch_words = [&](int c) {
+        w = load_words((iW ? s_fb : s_fa)[c / NCH] + ((c % NCH) * 256 + item) * 8);
+      };
+      fetch_words(0);
+      unsigned long long* near = reinterpret_cast<unsigned long long*>(smem);   // [n][2 TB] (the stages are idle)
+      bool look = false;
+      if (tid == 0) s_nfix = s_at = 0;
+#pragma unroll 2
       for (int i = tid; i < n * 2 * TB; i += NTHR) {
         const int e = i >> 7, q = i & 127;
-        s_ex[e][q] = (short)max(__ldcg((q < TB ? s_ea[e] : s_eb[e]) + (q & 63)), -32000);
+        const int4 row = __ldcg((q < TB ? s_ea[e] : s_eb[e]) + (q & 63));
+        s_ex[e][q] = (short)row.x;
+        near[i] = (unsigned)row.z | (unsigned long long)(unsigned)row.w << 32;
       }
       __syncthreads();
+      // every two rows share a near column (rows of zeros have all bits; both parts' threads hold the same
+      // outputs, so each looks at half of them)
+      if (!solve) {
+#pragma unroll 1
+        for (int e = 0; e < n; ++e) {
+          const uint2 b = *reinterpret_cast<const uint2*>(near + e * 2 * TB + TB + oc);
+          const uint4* a = reinterpret_cast<const uint4*>(near + e * 2 * TB + r0 + 8 * ri);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint4 v = a[i];
+            look |= ((v.x & b.x) | (v.y & b.y)) == 0 || ((v.z & b.x) | (v.w & b.y)) == 0;
+          }
+        }
+      }
       // the largest scale of every operand row over the task
       if (tid < 2 * TB) {
-        int m = -32000;
-        for (int e = 0; e < n; ++e) m = max(m, (int)s_ex[e][tid]);
+        int m = E_ZERO, lo = E_BAD;
+        for (int e = 0; e < n; ++e) {
+          m = max(m, (int)s_ex[e][tid]);
+          lo = min(lo, (int)s_ex[e][tid]);
+        }
         (tid < TB ? s_MA : s_MB)[tid & 63] = m;
+        look |= m > E_ZERO && lo < m - SPREAD / 2;
       }
-      __syncthreads();
-      const int nst = n * NCH;
+      const bool looked = __syncthreads_or(look || solve);
+      int nst = n * NCH;
+      if (looked) {
+        if (solve) {
+          const short2* old = reinterpret_cast<const short2*>(smem + OLD_OFF) + (PIV ? s_pm[oc] : oc);
+          const unsigned long long nb = near[TB + oc];
+          const int eb = s_MB[oc];
+#pragma unroll 2
+          for (int i = 0; i < 16; ++i) {
+            const short2 o = old[(r0 + i) * TB];
+            if (!(near[r0 + i] & nb) && max(o.x, o.y) - 1022 + SLACK < s_MA[r0 + i] + eb) fix |= 1u << i;
+          }
+        } else {
+          fix = short_outputs(s_ex, near, n, r0, oc, s_MA, s_MB);
+        }
+        if (fix) atomicAdd(&s_nfix, __popc(fix));
+        __syncthreads();
+        // most of them (over FIX_MAX of 8192): all by FMAs, which takes 0.6 of the list's time an output (groups above:
+        // half of the outputs 250 ms by the list, 312 all)
+        if (s_nfix > FIX_MAX) nst = 0;
+      }
       const uint32_t it0 = it, tile0 = tile_no;
       // one thread: the MMAs of stage c
       auto issue = [&](int c) {
@@ -449,11 +634,6 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         mma_commit(su(&bar_empty[s]));
         if (c % NCH == NCH - 1) mma_commit(su(&bar_accf));
       };
-      Words8 w;
-      auto fetch_words = [&](int c) {
-        w = load_words((iW ? s_fb : s_fa)[c / NCH] + ((c % NCH) * 256 + item) * 8);
-      };
-      fetch_words(0);
       // the first stage of a product is expanded before the read-back of the product before it, which
       // frees the tensor memory for its MMAs; the second one while those run
       for (int c = 0; c <= nst && !failed; ++c) {
@@ -490,10 +670,48 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         }
       }
       it = it0 + nst;
+      if (looked && s_nfix) {
+        const FixArgs g{p.tasks + task, p.klist, Lg, Linv, Dg, PIV ? reinterpret_cast<const double2*>(p.E) : nullptr, s_pm};
+        __syncthreads();                           // the last levels are read: the stages are free
+        if (nst == 0) {
+          fix = 0xffff;
+          const double2 *a = reinterpret_cast<const double2*>(smem) + r0 * LDS, *b = reinterpret_cast<const double2*>(smem + FIX_B) + oc * LDS;
+#pragma unroll 1
+          for (int e = 0; e < n; ++e) {
+            stage_operands(g, solve, e, smem);
+#pragma unroll
+            for (int i = 0; i < 16; i += 4) {
+              double v[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) v[u] = __longlong_as_double(H[i + u]);
+#pragma unroll 2
+              for (int k = 0; k < TB; ++k) {
+                const double2 w = part_of_b(b[k], ri);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = add_part(a[(i + u) * LDS + k], w, v[u]);
+              }
+#pragma unroll
+              for (int u = 0; u < 4; ++u) H[i + u] = __double_as_longlong(v[u]);
+            }
+            __syncthreads();
+          }
+        } else {
+          const int q0 = fix ? atomicAdd(&s_at, __popc(fix)) : 0;
+          int q = q0;
+#pragma unroll 1
+          for (unsigned f = fix; f; f &= f - 1) fix_list(smem)[q++] = (unsigned short)(ri << 12 | (r0 + __ffs(f) - 1) << 6 | oc);
+          __syncthreads();
+          fma_outputs(g, solve, n, smem, s_nfix);
+          q = q0;
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (fix >> i & 1) H[i] = __double_as_longlong(fix_sum(smem)[q++]);
+          __syncthreads();
+        }
+      }
     };
     auto result = [&](int i) -> double {
-      if (max(s_MA[r0 + i], s_MB[oc]) >= E_BAD) return __longlong_as_double(0x7ff8000000000000ll);
-      return fixed_to_double<28>(H[i], Lo[i], s_MA[r0 + i] + s_MB[oc] - 74);
+      return fix >> i & 1 ? __longlong_as_double(H[i]) : fixed_to_double<28>(H[i], Lo[i], s_MA[r0 + i] + s_MB[oc] - 74);
     };
 
     // ---------------------------------------------------------------- 1. Schur products
@@ -506,7 +724,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         s_eb[tid] = EW + (int64_t)ke.b_tile * TB;
       }
       __syncthreads();
-      products(T.nk);
+      products(T.nk, false);
     }
     if (__syncthreads_or(failed)) {
       if (tid == 0) set_error(p.ctl, D3M_ERR_TIMEOUT, task);
@@ -593,23 +811,33 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         constexpr int NR = decltype(nrow)::value;
         if (iW || irow < NR) {
           double v[8];
-          int m = X_ZERO;
-          const int sg = iW ? -1 : 1;
+          int m = X_ZERO, sh[8], ex[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const int q = ik8 * 8 + e;
             v[e] = value(iW, irow, q, ipart);
-            m = max(m, exp_of(v[e], sg * s_ek[c0 + q]));
+            sh[e] = iW ? -s_ek[c0 + q] : s_ek[c0 + q];
+            ex[e] = exp_of(v[e], sh[e]);
+            m = max(m, ex[e]);
           }
           m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
           m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
           const int E = row_scale(m);
-          if ((item & 3) == 0) (iW ? s_MB : s_MA)[irow] = E;
+          unsigned nb = 0;                        // the row's columns near its largest entry
+#pragma unroll
+          for (int e = 0; e < 8; ++e) nb |= (unsigned)near_max(ex[e], m) << e;
+          nb <<= ik8 * 8;
+          nb |= __shfl_xor_sync(0xffffffffu, nb, 1);
+          nb |= __shfl_xor_sync(0xffffffffu, nb, 2);
+          if ((item & 3) == 0) {
+            (iW ? s_MB : s_MA)[irow] = E;
+            (iW ? s_nearW : s_nearL)[irow] = (unsigned short)(no_near(E) ? 0 : nb);
+          }
           Words8 w;
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            w.w[e].x = word_of(v[2 * e], sg * s_ek[c0 + ik8 * 8 + 2 * e], E);
-            w.w[e].y = word_of(v[2 * e + 1], sg * s_ek[c0 + ik8 * 8 + 2 * e + 1], E);
+            w.w[e].x = word_of(v[2 * e], sh[2 * e], E);
+            w.w[e].y = word_of(v[2 * e + 1], sh[2 * e + 1], E);
           }
           put_digits<NR>(smem, iW, irow, ipart, ik8, w);
         }
@@ -629,6 +857,17 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         fence_after();
 #pragma unroll
         for (int i = 0; i < 16; ++i) H[i] = Lo[i] = 0;
+      };
+      // output (r, oc) of a local product, a term of a sum that starts at `old`: whether it needs FMAs, and their sum
+      auto local_short = [&](int r, double old) -> bool {
+        return !(s_nearL[r] & s_nearW[oc]) && exp_of(old, 0) - 1022 + SLACK < s_MA[r] + s_MB[oc];
+      };
+      auto local_fma = [&](int r, auto value) -> double {
+        double s = 0.0;
+#pragma unroll 1
+        for (int q = 0; q < PW; ++q)
+          s = add_part(make_double2(value(false, r, q, 0), value(false, r, q, 1)), part_of_b(make_double2(value(true, oc, q, 0), value(true, oc, q, 1)), ri), s);
+        return s;
       };
       auto product_read = [&]() {
         fence_before();
@@ -714,21 +953,30 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         __syncthreads();
         const int c1 = c0 + PW;
         // V = sS[:, panel] X_kk^T, rows outside the panel: the W side holds the 64 rows, the L side
-        // X_kk, so a thread reads back 4 columns of row oc
-        local_product(I16{}, c0, [&](bool ws, int row, int q, int part) -> double {
-          if (!ws) return reinterpret_cast<const double*>(&sX[row][q])[part];
+        // X_kk without its diagonal, so a thread reads back 4 columns of row oc
+        auto v_value = [&](bool ws, int row, int q, int part) -> double {
+          if (!ws) return row != q ? reinterpret_cast<const double*>(&sX[row][q])[part] : 0.0;
           return (row < c0 || row >= c1) ? reinterpret_cast<const double*>(sS + row * LDS + c0 + q)[part] : 0.0;
-        });
+        };
+        local_product(I16{}, c0, v_value);
         if (failed) break;
         {
           const int q0 = (warp >> 2) * 4;
           read_levels(I4{}, I16{}, q0, [](int) { return 0; });
           product_read();
-          const int m = max(max(s_MA[q0], s_MA[q0 + 1]), max(max(s_MA[q0 + 2], s_MA[q0 + 3]), s_MB[oc]));
+          const double* old = reinterpret_cast<const double*>(sS + oc * LDS + c0 + q0) + ri;
+          double* v = sV + (ri * TB + oc) * (PW + 1) + q0;
+          unsigned fl = 0;
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            sV[(ri * TB + oc) * (PW + 1) + q0 + i] =
-                m >= E_BAD ? __longlong_as_double(0x7ff8000000000000ll) : fixed_to_double<28>(H[i], Lo[i], s_MA[q0 + i] + s_MB[oc] - 74);
+          for (int i = 0; i < 4; ++i) {
+            v[i] = old[2 * i] + fixed_to_double<28>(H[i], Lo[i], s_MA[q0 + i] + s_MB[oc] - 74);
+            if (local_short(q0 + i, old[2 * i])) fl |= 1u << i;
+          }
+#pragma unroll 1
+          for (; fl; fl &= fl - 1) {
+            const int i = __ffs(fl) - 1;
+            v[i] = old[2 * i] + local_fma(q0 + i, v_value);
+          }
         }
         __syncthreads();
         // above the panel X = -V, below L = V / d
@@ -740,11 +988,13 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         }
         __syncthreads();
         if (c1 >= nr) break;
-        local_product(I64{}, c0, [&](bool ws, int row, int q, int part) -> double {
+        // (U inside the panel without the diagonal of -X_kk: L[r][s] itself is added to Z[r][s], which is zero there)
+        auto t_value = [&](bool ws, int row, int q, int part) -> double {
           if (!ws) return row >= c1 ? reinterpret_cast<const double*>(sS + row * LDS + c0 + q)[part] : 0.0;
           if (row < c0 || row >= c1) return sV[(part * TB + row) * (PW + 1) + q];
-          return -reinterpret_cast<const double*>(&sX[q][row - c0])[part];
-        });
+          return q != row - c0 ? -reinterpret_cast<const double*>(&sX[q][row - c0])[part] : 0.0;
+        };
+        local_product(I64{}, c0, t_value);
         if (failed) break;
         // rows c1 .. 63 in groups of 4, a quarter of them to each of the four warps of an SM partition
         {
@@ -754,15 +1004,23 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
 #pragma unroll
             for (int i = 0; i < 4; ++i) H[i] = Lo[i] = 0;
             read_levels(I4{}, I64{}, rb, [](int) { return 0; });
+            unsigned fl = 0;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               const int r = rb + i;
               if (oc <= r) {
-                const double v = max(s_MA[r], s_MB[oc]) >= E_BAD ? __longlong_as_double(0x7ff8000000000000ll)
-                                                                   : fixed_to_double<28>(H[i], Lo[i], s_MA[r] + s_MB[oc] - 74);
                 double* t = reinterpret_cast<double*>(oc >= c1 ? sS + r * LDS + oc : sS + oc * LDS + r) + ri;
-                *t -= v;
+                const double old = oc >= c0 && oc < c1 ? reinterpret_cast<const double*>(sS + r * LDS + oc)[ri] : *t;
+                if (!local_short(r, old)) *t = old - fixed_to_double<28>(H[i], Lo[i], s_MA[r] + s_MB[oc] - 74);
+                else fl |= 1u << i;
               }
+            }
+#pragma unroll 1
+            for (; fl; fl &= fl - 1) {
+              const int r = rb + __ffs(fl) - 1;
+              double* t = reinterpret_cast<double*>(oc >= c1 ? sS + r * LDS + oc : sS + oc * LDS + r) + ri;
+              const double old = oc >= c0 && oc < c1 ? reinterpret_cast<const double*>(sS + r * LDS + oc)[ri] : *t;
+              *t = old - local_fma(r, t_value);
             }
           }
         }
@@ -798,23 +1056,28 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         for (int i = 0; i < 4; ++i) {
           const int r = warp + 16 * i;
           double2 x[2];
-          int m = X_ZERO;
+          int m = X_ZERO, ex[2];
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             const int s = lane + 32 * q;
-            x[q] = (s < r && (PIV || r < nr)) ? sS[s * LDS + r] : make_double2(s == r ? 1.0 : 0.0, 0.0);
-            m = max(m, max(exp_of(x[q].x, s_ek[s]), exp_of(x[q].y, s_ek[s])));
+            x[q] = (s < r && (PIV || r < nr)) ? sS[s * LDS + r] : make_double2(0.0, 0.0);
+            ex[q] = max(exp_of(x[q].x, s_ek[s]), exp_of(x[q].y, s_ek[s]));
+            m = max(m, ex[q]);
           }
           m = __reduce_max_sync(0xffffffffu, m);
           const int E = row_scale(m);
-          if (lane == 0) EL[(int64_t)T.tile * TB + r] = E;
+          unsigned near0 = 0, near1 = 0;
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
-            const int s = lane + 32 * q, k = PIV ? s_bk.perm[s] : s;   // column k of X = Lt^{-1}
-            Li[r * TB + k] = x[q];
+            const int s = lane + 32 * q, k = PIV ? s_bk.perm[s] : s;   // column k of X = Lt^{-1}; words without its diagonal
+            Li[r * TB + k] = s == r ? make_double2(1.0, 0.0) : x[q];
             f[word_at(r, k, 0)] = word_of(x[q].x, s_ek[s], E);
             f[word_at(r, k, 1)] = word_of(x[q].y, s_ek[s], E);
+            if (near_max(ex[q], m)) (k < 32 ? near0 : near1) |= 1u << (k & 31);
           }
+          near0 = __reduce_or_sync(0xffffffffu, near0);
+          near1 = __reduce_or_sync(0xffffffffu, near1);
+          if (lane == 0) EL[(int64_t)T.tile * TB + r] = row_info(m, near0, near1);
         }
         double2* Lt = Lg + (int64_t)T.tile * TB * TB;
         for (int i = tid; i < TB * TB; i += NTHR) {
@@ -854,11 +1117,12 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
       }
     } else {
       // -------------------------------------------------------------- 2b. off-diagonal tile
-      // W_IJ = S X^T with the words of S in this tile's own slot, then L_IJ = W_IJ / d
+      // W_IJ = S X^T = S + S (X - I)^T with the words of S in this tile's own slot, then L_IJ = W_IJ / d
       unsigned long long* f = FL + (int64_t)T.tile * TW;
       if (tid < TB) {
         s_eL[tid] = X_ZERO;
         s_eW[tid] = X_ZERO;
+        s_near[tid][0] = s_near[tid][1] = 0;
         const double2 d = ld_cg(Dg + (int64_t)T.col * TB + tid);
         s_d[tid] = d;
         if constexpr (PIV) {
@@ -876,7 +1140,8 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
           const int bal = pair_balance(d, o, first2 || second2 ? e : d);
           s_ek[tid] = bal;
           // the contraction of the triangular solve runs over the tile's own order
-          s_eS[p.piv[(int64_t)T.col * TB + tid]] = bal;
+          s_pm[tid] = p.piv[(int64_t)T.col * TB + tid];
+          s_eS[s_pm[tid]] = bal;
         } else {
           s_ek[tid] = s_eS[tid] = balance_of(d);
           s_rec[tid] = 1.0 / (d.x * d.x + d.y * d.y);
@@ -892,11 +1157,20 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
         }
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 16; ++i) f[word_at(r0 + i, oc, ri)] = word_of(S[i], -bal, row_scale(s_eL[r0 + i]));
+        for (int i = 0; i < 16; ++i) {
+          const int m = s_eL[r0 + i];
+          f[word_at(r0 + i, oc, ri)] = word_of(S[i], -bal, row_scale(m));
+          if (!s_in) Sa[ri * TB * TB + (r0 + i) * TB + oc] = S[i];   // read again after the product
+          reinterpret_cast<short*>(smem + OLD_OFF)[((r0 + i) * TB + oc) * 2 + ri] = (short)exp_of(S[i], 0);
+          const unsigned near = __ballot_sync(0xffffffffu, near_max(exp_of(S[i], -bal), m));
+          if (lane == 0) atomicOr(&s_near[r0 + i][warp & 1], near);
+        }
       }
-      if (tid < TB) EL[(int64_t)T.tile * TB + tid] = row_scale(s_eL[tid]);
       __syncthreads();
-      if (tid < TB) s_eL[tid] = X_ZERO;
+      if (tid < TB) {
+        EL[(int64_t)T.tile * TB + tid] = row_info(s_eL[tid], s_near[tid][0], s_near[tid][1]);
+        s_eL[tid] = X_ZERO;
+      }
       if (tid == 0) {
         s_fa[0] = f;
         s_fb[0] = FL + (int64_t)T.diag * TW;
@@ -905,14 +1179,14 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
       }
       __syncthreads();
       trace_mark(p, task, 1);
-      products(1);
+      products(1, true);
       if (__syncthreads_or(failed)) {
         if (tid == 0) set_error(p.ctl, D3M_ERR_TIMEOUT, task);
         break;
       }
       {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) sW[(ri * TB + r0 + i) * LDS + oc] = result(i);
+        for (int i = 0; i < 16; ++i) sW[(ri * TB + r0 + i) * LDS + oc] = __ldcg(Sa + ri * TB * TB + (r0 + i) * TB + (PIV ? s_pm[oc] : oc)) + result(i);
       }
       __syncthreads();
       trace_mark(p, task, 2);
@@ -953,10 +1227,17 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
           f[word_at(r, c, 1)] = word_of(l[i].y, bal, eL);
           g[word_at(r, c, 0)] = word_of(w[i].x, -bal, eW);
           g[word_at(r, c, 1)] = word_of(w[i].y, -bal, eW);
+          const unsigned nl = __ballot_sync(0xffffffffu, near_max(max(exp_of(l[i].x, bal), exp_of(l[i].y, bal)), s_eL[r]));
+          const unsigned nw = __ballot_sync(0xffffffffu, near_max(max(exp_of(w[i].x, -bal), exp_of(w[i].y, -bal)), s_eW[r]));
+          if (lane == 0) {
+            s_near[r][warp & 1] = nl;
+            s_nearV[r][warp & 1] = nw;
+          }
         }
+        __syncthreads();
         if (tid < TB) {
-          EL[(int64_t)T.tile * TB + tid] = row_scale(s_eL[tid]);
-          EW[(int64_t)T.tile * TB + tid] = row_scale(s_eW[tid]);
+          EL[(int64_t)T.tile * TB + tid] = row_info(s_eL[tid], s_near[tid][0], s_near[tid][1]);
+          EW[(int64_t)T.tile * TB + tid] = row_info(s_eW[tid], s_nearV[tid][0], s_nearV[tid][1]);
         }
       }
     }
