@@ -43,11 +43,6 @@ def fp64_peak(info, peaks):
     return "alu", FP64_FMA_TFLOPS, "FP64 FMA 152 SMs x 2 x 2 x 2.07 GHz"
 
 
-# the residual's products issue on the FP32 pipe in double-float form: 60 FP32 instructions per
-# complex multiply-add (8 flops) and right-hand side
-RESID_PEAK_TFLOPS = 152 * 128 * 2.07e9 * 8 / 60 / 1e12
-
-
 def parse_args():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)

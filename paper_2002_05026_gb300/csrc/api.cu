@@ -451,7 +451,7 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
   }
   if (h->opt.pivot && h->tc) {
     delete h;
-    return set_err(nullptr, D3M_ERR_INVALID, "pivoting needs a SIMT engine (D3M_FP64 or D3M_MIXED_SIMT32)");
+    return set_err(nullptr, D3M_ERR_INVALID, "pivoting needs D3M_FP64 or D3M_MIXED_SIMT32");
   }
   if (h->fp64 && (h->opt.fp64_engine < D3M_FP64_AUTO || h->opt.fp64_engine > D3M_FP64_FMA)) {
     delete h;
@@ -461,7 +461,9 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
   // mixed precision: a tile's Schur updates from up to 8 source blocks form one update task (the
   // per-task epilogue through the accumulator dominates short segments), 32 with TF32 (its
   // factorization is bound by DRAM, and every segment boundary writes and reads back the tile's
-  // accumulator); FP64 is DFMA bound and keeps one task per source block
+  // accumulator); FP64 keeps one task per source block, the earliest start: its update tasks are long (10 us a
+  // product) and small systems wait for their chain (3 x 3 blocks of 100: factorization 2.99 ms, 3.44 with 8; 4 x 4
+  // of 512: 21.4, 21.0 with 2, 21.4 with 8)
   if (h->opt.seg_group <= 0) h->opt.seg_group = h->fp64 ? 1 : (h->tf32 ? 32 : 8);
   // the tensor-core gathers of the solve (split-BF16x3 products, both engines) sum up to 16 items of one
   // destination in tensor memory

@@ -56,7 +56,7 @@ struct FactorParams {
   int64_t* trace;        // [ntasks][8] task records, or nullptr
   int64_t timeout_ns;
   double piv_tol;        // breakdown: |d| < piv_tol * max|S| of the diagonal tile
-  int pivot;             // 1: Bunch-Kaufman pivoting inside diagonal tiles (SIMT engine)
+  int pivot;             // 1: Bunch-Kaufman pivoting inside diagonal tiles (SIMT and FP64 digit engines)
   void* E;               // [NT][b] sub-diagonal entry of each 2 x 2 pivot block (pivot mode), 0 else
   int32_t* piv;          // [NT][b] permutation of each diagonal tile (pivot mode)
 };

@@ -306,7 +306,8 @@ __device__ __forceinline__ double mul_part(double2 u, double2 z, int p) {
 // into FP32's range (relative error r of about 2^-23), then y (1 + r + r^2) with r = 1 - d y in FP64 and
 // r^2 in FP32 (the dropped r^3 is 2^-69).  An FP64 instruction of a warp takes 64 cycles of its SM
 // partition whatever the lanes do: five of them here, a complex division is sixteen.  Pivots
-// outside 2^(+-1000), zeros, Inf and NaN take the division.
+// outside 2^(+-1000), zeros, Inf and NaN take the division.  (The off-diagonal tiles, like the sweeps and the FMA
+// engine, divide by d through |d|^2, which needs |d| within 2^(+-511).)
 __device__ __forceinline__ double recip_part(double dp, int p) {
   const double dq = shfl_d(dp, 1);
   const double dx = p ? dq : dp, dy = p ? dp : dq;

@@ -103,7 +103,7 @@ int resid_tc_groups(int nrhs, int* NR);
 int launch_resid_tc(const ResidualTc& p, const double2* X, const double2* B, double2* R,
                     int nrhs, int nrtiles, int nblk, int max_rtiles, cudaStream_t st, int64_t* launches);
 
-// FP64 (unpivoted) with the tile products as exact digit products on the tensor cores
+// FP64 with the tile products as digit products on the tensor cores, with or without pivoting
 constexpr int kDigMaxProducts = 64;    // most tile products of one task
 int launch_factor_dig(const FactorParams& p, int nblocks, cudaStream_t st);
 int launch_factor_simt(const FactorParams& p, bool fp64, int nblocks, cudaStream_t st);

@@ -1010,8 +1010,9 @@ constexpr int CHAIN_MAXJ = 128;   // staged strips of one CTA
 constexpr int CHAIN_MAXCL = 8;    // portable cluster size
 constexpr int CHAIN_MAXLOC = 4;   // strips per CTA
 // Partials per row above which a level gets a separate reduce launch: the chain subtracts fewer itself, sixteen
-// loads in flight a thread, in less time than a launch takes (at 12: 6.3 ms of sweeps on a 5 x 5 x 3 grid, m = 256,
-// 32 right-hand sides, at 80 6.0 ms; 8 x 8, m = 512: 3.82, 3.78 at 32, 3.85 at 80).
+// loads in flight a thread, in less time than a launch takes.  Milliseconds of a sweep at 12, 32, 48 and 80 (runs of
+// one setting differ by under 0.5 %): 5 x 5 x 3 grid, m = 256, 32 right-hand sides 2.88, 2.71, 2.66, 2.66; 5 x 5 x 4, m = 512,
+// 32: 9.27, 9.12, 9.09, 9.11; 64 uneven systems 1.54, 1.50, 1.49, 1.49; 8 x 8, m = 512, 8: 1.76, 1.74, 1.75, 1.77.
 constexpr int EXT_REDUCE = 48;
 
 // INV mode: the diagonal block is applied as one product with its stored inverse,
