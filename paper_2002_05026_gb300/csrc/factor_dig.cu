@@ -27,10 +27,12 @@
 // exponent.  Two rows that share one have sum |a_k b_k| >= 2^-6 of the scales' product; an output whose rows share
 // none (or whose scales lie 2^13 below those of the task's largest product, or near the subnormal numbers, or in
 // rows with an Inf or NaN) is formed by FP64 FMAs (fma_outputs).  X_JJ and a panel's X_kk are held without their
-// unit diagonal, whose term is added in FP64: it would set the scale of every row of a dominant tile.  Error of the
-// worst of the groups of unknowns of a dense system, coupled by eps^|g_i - g_j| and driven in one of them (digits
-// alone, digits and FMAs, FMAs alone): two groups, eps = 1e-4: 1.7e-12, 4.8e-16, 7.9e-16; 1e-8: 1.7e-8, 3.5e-16,
-// 6.2e-16; eight groups, eps = 2^-4: 2.4e-8, 1.6e-15, 7e-16; no groups: 4.9e-16, 4.1e-16, 7.1e-16.
+// unit diagonal, whose term is added in FP64: it would set the scale of every row of a dominant tile; beside it a
+// product may be short if 2^SLACK of the term reaches the scales'.  Error of the worst of the groups of unknowns of a
+// dense system, coupled by eps^|g_i - g_j| and driven in one of them, largest of three draws (digits alone, digits
+// and FMAs, FMAs alone): two groups, eps = 1e-4: 1.7e-12, 4.1e-16, 7.9e-16; 1e-8: 1.7e-8, 3.6e-16, 6.2e-16; eight groups, eps
+// = 2^-4: 2.4e-8, 4.9e-16, 7.4e-16 (SLACK = 6: 2.1e-15; with pivoting 6.2e-16 and 6.2e-16); eps = 1 / 2: - , 5.2e-16,
+// 7.6e-16; no groups: 4.9e-16, 4.1e-16, 7.1e-16.
 // Cost, 4 x 4 grid, m = 512: dense: 2 % of the tasks have a few such outputs, factorization 20.2 -> 21.4 ms (an update
 // of eight products 104 -> 106 us, an off-diagonal tile 44 -> 51, a diagonal one 162 -> 172); two and eight groups:
 // 250 and 310 ms (FMAs alone: 255).
@@ -160,7 +162,7 @@ __device__ __forceinline__ int4 row_info(int rowmax, unsigned lo, unsigned hi) {
   const int E = row_scale(rowmax);
   return no_near(E) ? make_int4(E, 0, 0, 0) : make_int4(E, 0, (int)lo, (int)hi);
 }
-constexpr int SLACK = 6;                         // a term beside a product counts if 2^SLACK of it reaches the scales'
+constexpr int SLACK = 3;                         // see the top
 constexpr int SPREAD = 13;                       // bits of the fixed-point sum past a product's own
 constexpr int E_NONE = -100000;
 // biased word of x 2^shift for scale 2^E (|x 2^shift| < 2^E): bytes 6..0 = digits 0..6 plus 128
