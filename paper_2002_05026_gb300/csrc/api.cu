@@ -68,6 +68,8 @@ struct d3m_ctx {
   void* opS = nullptr;               // TF32: bf16 split planes of L for the solve's tensor-core products
   int4* rowA = nullptr;              // digit engine: row scales of opA / opB and the columns near them
   int4* rowB = nullptr;
+  uint2* nzA = nullptr;              // and their nonzero columns
+  uint2* nzB = nullptr;
   void* Sacc = nullptr;
   void* E = nullptr;                 // pivot mode: sub-diagonals of the 2 x 2 pivot blocks [NT][b]
   int32_t* piv = nullptr;            // pivot mode: permutation of every diagonal tile [NT][b]
@@ -804,11 +806,13 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
       h->opB = dalloc<unsigned char>(h, words);
       h->rowA = dalloc<int4>(h, rows);
       h->rowB = dalloc<int4>(h, rows);
-      h->dig = h->opA && h->opB && h->rowA && h->rowB;
+      h->nzA = dalloc<uint2>(h, rows);
+      h->nzB = dalloc<uint2>(h, rows);
+      h->dig = h->opA && h->opB && h->rowA && h->rowB && h->nzA && h->nzB;
       if (!h->dig) {
-        void* part[4] = {h->opA, h->opB, h->rowA, h->rowB};
-        const size_t bytes[4] = {words, words, rows * sizeof(int4), rows * sizeof(int4)};
-        for (int q = 0; q < 4; ++q)
+        void* part[6] = {h->opA, h->opB, h->rowA, h->rowB, h->nzA, h->nzB};
+        const size_t bytes[6] = {words, words, rows * sizeof(int4), rows * sizeof(int4), rows * sizeof(uint2), rows * sizeof(uint2)};
+        for (int q = 0; q < 6; ++q)
           if (part[q]) {
             h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), part[q]));
             h->dev_bytes -= (int64_t)bytes[q];
@@ -816,6 +820,7 @@ static int create_impl(d3m_handle* out, const d3m_pattern* pat, const int32_t* p
           }
         h->opA = h->opB = nullptr;
         h->rowA = h->rowB = nullptr;
+        h->nzA = h->nzB = nullptr;
         if (want == D3M_FP64_DIGITS) return set_err(h, D3M_ERR_OOM, "cudaMalloc failed for the digit words");
       }
     }
@@ -978,6 +983,8 @@ static int enqueue_factor(d3m_ctx* h, const void* Kin, bool kdev, cudaStream_t s
   p.opS = h->opS;
   p.rowA = h->rowA;
   p.rowB = h->rowB;
+  p.nzA = h->nzA;
+  p.nzB = h->nzB;
   p.k_arrived = kup ? h->k_arrived : nullptr;
   p.Sacc = h->Sacc;
   p.trace = h->trace;

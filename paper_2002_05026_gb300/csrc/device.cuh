@@ -50,6 +50,8 @@ struct FactorParams {
   void* opB;             // tensor-core operand planes (bf16) of W tiles / T_J; FP64: digit words of W
   int4* rowA;            // FP64 digit engine: rows of opA, opB [ntiles][b]: scale, columns near the largest entry
   int4* rowB;
+  uint2* nzA;            // the same rows' nonzero columns
+  uint2* nzB;
   void* opS;             // TF32 engine: bf16 split planes of the L tiles for the solve's products, or nullptr
   const int32_t* k_arrived;  // upload progress of a host K (stored blocks in upload order), or nullptr
   void* Sacc;            // [n_acc][b][b] partial Schur accumulators (tensor-core c64 engines; the others use L's tiles)

@@ -26,7 +26,8 @@
 // which the balance removes.  Every row therefore carries its near columns, those within 2^-2 of its largest
 // exponent.  Two rows that share one have sum |a_k b_k| >= 2^-6 of the scales' product; an output whose rows share
 // none (or whose scales lie 2^13 below those of the task's largest product, or near the subnormal numbers, or in
-// rows with an Inf or NaN) is formed by FP64 FMAs (fma_outputs).  X_JJ and a panel's X_kk are held without their
+// rows with an Inf or NaN) is formed by FP64 FMAs (fma_outputs), unless its rows meet in zeros only, which the
+// nonzero columns of a row tell: two uncoupled groups of unknowns 24 ms instead of 253.  X_JJ and a panel's X_kk are held without their
 // unit diagonal, whose term is added in FP64: it would set the scale of every row of a dominant tile; beside it a
 // product may be short if 2^SLACK of the term reaches the scales'.  Error of the worst of the groups of unknowns of a
 // dense system, coupled by eps^|g_i - g_j| and driven in one of them, largest of three draws (digits alone, digits
@@ -34,7 +35,7 @@
 // = 2^-4: 2.4e-8, 4.9e-16, 7.4e-16 (SLACK = 6: 2.1e-15; with pivoting 6.2e-16 and 6.2e-16); eps = 1 / 2: - , 5.2e-16,
 // 7.6e-16; no groups: 4.9e-16, 4.1e-16, 7.1e-16.
 // Cost, 4 x 4 grid, m = 512: dense: 2 % of the tasks have a few such outputs, factorization 20.2 -> 21.4 ms (an update
-// of eight products 104 -> 106 us, an off-diagonal tile 44 -> 51, a diagonal one 162 -> 172); two and eight groups:
+// of eight products 104 -> 106 us, an off-diagonal tile 44 -> 52, a diagonal one 162 -> 172); two and eight groups:
 // 250 and 310 ms (FMAs alone: 255).
 //
 // One product: MMA M = 128 rows [Re c | Im c] of the embedded W (rows [b_r | -b_i], then
@@ -158,6 +159,10 @@ constexpr int NEAR = 2;
 __device__ __forceinline__ int row_scale(int be) { return be >= X_BAD ? E_BAD : max(be - 1022, E_ZERO); }
 __device__ __forceinline__ bool near_max(int e, int rowmax) { return e >= rowmax - NEAR; }
 __device__ __forceinline__ bool no_near(int E) { return E >= E_BAD || (E < E_TINY && E > E_ZERO); }
+// its nonzero columns; all for a row of zeros or with an Inf or NaN, so that the two meet
+__device__ __forceinline__ uint2 row_nonzero(int rowmax, unsigned lo, unsigned hi) {
+  return rowmax <= X_ZERO || rowmax >= X_BAD ? make_uint2(~0u, ~0u) : make_uint2(lo, hi);
+}
 __device__ __forceinline__ int4 row_info(int rowmax, unsigned lo, unsigned hi) {
   const int E = row_scale(rowmax);
   return no_near(E) ? make_int4(E, 0, 0, 0) : make_int4(E, 0, (int)lo, (int)hi);
@@ -337,19 +342,21 @@ __device__ __forceinline__ double recip_part(double dp, int p) {
   return scale2(t, k);
 }
 
-// Outputs of an update whose digit sum would fall short of FP64 (bit i: output (r0 + i, c)): ex, near: scales and near
-// columns of the n products' rows [n][2 TB]
-__device__ __noinline__ unsigned short_outputs(const short (*ex)[2 * TB], const unsigned long long* near, int n, int r0, int c,
-                                               const int* MA, const int* MB) {
+// Outputs of an update whose digit sum would fall short of FP64 (bit i: output (r0 + i, c)): ex, near, nz: scales, near
+// and nonzero columns of the n products' rows [n][2 TB]
+__device__ __noinline__ unsigned short_outputs(const short (*ex)[2 * TB], const unsigned long long* near, const unsigned long long* nz,
+                                               int n, int r0, int c, const int* MA, const int* MB) {
   unsigned fix = 0;
 #pragma unroll 1
   for (int i = 0; i < 16; ++i) {
     int best = E_NONE, rest = E_NONE;              // largest product of scales with a column near both, without
+#pragma unroll 2
     for (int e = 0; e < n; ++e) {
+      const int a = e * 2 * TB + r0 + i, b = e * 2 * TB + TB + c;
       const int ea = ex[e][r0 + i], eb = ex[e][TB + c];
-      const bool hit = (near[e * 2 * TB + r0 + i] & near[e * 2 * TB + TB + c]) != 0;
-      if (!hit) rest = max(rest, ea + eb);
-      else if (min(ea, eb) > E_ZERO) best = max(best, ea + eb);
+      const bool hit = (near[a] & near[b]) != 0;
+      if (hit && min(ea, eb) > E_ZERO) best = max(best, ea + eb);
+      if (!hit && (nz[a] & nz[b])) rest = max(rest, ea + eb);       // rows that meet in zeros only: exactly zero
     }
     if (rest > best || (best > E_NONE && MA[r0 + i] + MB[c] - best > SPREAD)) fix |= 1u << i;
   }
@@ -459,7 +466,8 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
   __shared__ short s_ex[MAXP][2 * TB];            // row scales of every product of the task
   __shared__ int s_eL[TB], s_eW[TB];              // largest biased exponents of finished rows
   __shared__ unsigned s_near[TB][2], s_nearV[TB][2];   // columns near them (L or S, W)
-  __shared__ unsigned short s_nearL[TB], s_nearW[TB];   // the same of a panel product's operands
+  __shared__ unsigned s_nz[TB][2], s_nzV[TB][2];  // nonzero columns
+  __shared__ unsigned s_nearL[TB], s_nearW[TB];   // the same of a panel product's operands: near, nonzero << 16
   __shared__ int s_pm[TB];                        // pivot mode: the tile's own order
   __shared__ int s_nfix, s_at;                    // short outputs of a task; listed so far
   __shared__ int s_ek[TB], s_eS[TB];              // balance of every column; the same in the tile's order
@@ -478,6 +486,8 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
   unsigned long long* FW = reinterpret_cast<unsigned long long*>(p.opB);
   int4* EL = p.rowA;
   int4* EW = p.rowB;
+  uint2* ZL = p.nzA;
+  uint2* ZW = p.nzB;
   constexpr int64_t TW = 2 * TB * TB;             // words of a tile
 
   if (tid == 0) {
@@ -572,6 +582,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
       unsigned long long* near = reinterpret_cast<unsigned long long*>(smem);   // [n][2 TB] (the stages are idle)
       bool look = false;
       if (tid == 0) s_nfix = s_at = 0;
+      const uint2 zx = solve ? __ldcg(ZL + (s_eb[0] - EL) + oc) : make_uint2(0, 0);   // nonzero columns of row oc of X_JJ
 #pragma unroll 2
       for (int i = tid; i < n * 2 * TB; i += NTHR) {
         const int e = i >> 7, q = i & 127;
@@ -614,10 +625,18 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
 #pragma unroll 2
           for (int i = 0; i < 16; ++i) {
             const short2 o = old[(r0 + i) * TB];
-            if (!(near[r0 + i] & nb) && max(o.x, o.y) - 1022 + SLACK < s_MA[r0 + i] + eb) fix |= 1u << i;
+            const bool meet = (s_nz[r0 + i][0] & zx.x) | (s_nz[r0 + i][1] & zx.y);
+            if (!(near[r0 + i] & nb) && meet && max(o.x, o.y) - 1022 + SLACK < s_MA[r0 + i] + eb) fix |= 1u << i;
           }
         } else {
-          fix = short_outputs(s_ex, near, n, r0, oc, s_MA, s_MB);
+          unsigned long long* nz = reinterpret_cast<unsigned long long*>(smem + OLD_OFF);   // [n][2 TB]
+          for (int i = tid; i < n * 2 * TB; i += NTHR) {
+            const int e = i >> 7, q = i & 127;
+            const uint2 z = __ldcg(q < TB ? ZL + (s_ea[e] - EL) + q : ZW + (s_eb[e] - EW) + q - TB);
+            nz[i] = z.x | (unsigned long long)z.y << 32;
+          }
+          __syncthreads();
+          fix = short_outputs(s_ex, near, nz, n, r0, oc, s_MA, s_MB);
         }
         if (fix) atomicAdd(&s_nfix, __popc(fix));
         __syncthreads();
@@ -828,13 +847,13 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
           const int E = row_scale(m);
           unsigned nb = 0;                        // the row's columns near its largest entry
 #pragma unroll
-          for (int e = 0; e < 8; ++e) nb |= (unsigned)near_max(ex[e], m) << e;
+          for (int e = 0; e < 8; ++e) nb |= ((unsigned)near_max(ex[e], m) | (unsigned)(ex[e] != X_ZERO) << 16) << e;
           nb <<= ik8 * 8;
           nb |= __shfl_xor_sync(0xffffffffu, nb, 1);
           nb |= __shfl_xor_sync(0xffffffffu, nb, 2);
           if ((item & 3) == 0) {
             (iW ? s_MB : s_MA)[irow] = E;
-            (iW ? s_nearW : s_nearL)[irow] = (unsigned short)(no_near(E) ? 0 : nb);
+            (iW ? s_nearW : s_nearL)[irow] = no_near(E) ? (nb & 0xffff0000u) | (E >= E_BAD ? 0xffff0000u : 0) : (m <= X_ZERO ? ~0u : nb);
           }
           Words8 w;
 #pragma unroll
@@ -863,7 +882,8 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
       };
       // output (r, oc) of a local product, a term of a sum that starts at `old`: whether it needs FMAs, and their sum
       auto local_short = [&](int r, double old) -> bool {
-        return !(s_nearL[r] & s_nearW[oc]) && exp_of(old, 0) - 1022 + SLACK < s_MA[r] + s_MB[oc];
+        const unsigned both = s_nearL[r] & s_nearW[oc];     // rows that meet in zeros only: exactly zero
+        return both >= 0x10000u && !(both & 0xffffu) && exp_of(old, 0) - 1022 + SLACK < s_MA[r] + s_MB[oc];
       };
       auto local_fma = [&](int r, auto value) -> double {
         double s = 0.0;
@@ -1069,7 +1089,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
           }
           m = __reduce_max_sync(0xffffffffu, m);
           const int E = row_scale(m);
-          unsigned near0 = 0, near1 = 0;
+          unsigned near0 = 0, near1 = 0, nz0 = 0, nz1 = 0;
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             const int s = lane + 32 * q, k = PIV ? s_bk.perm[s] : s;   // column k of X = Lt^{-1}; words without its diagonal
@@ -1077,10 +1097,16 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
             f[word_at(r, k, 0)] = word_of(x[q].x, s_ek[s], E);
             f[word_at(r, k, 1)] = word_of(x[q].y, s_ek[s], E);
             if (near_max(ex[q], m)) (k < 32 ? near0 : near1) |= 1u << (k & 31);
+            if (ex[q] != X_ZERO) (k < 32 ? nz0 : nz1) |= 1u << (k & 31);
           }
           near0 = __reduce_or_sync(0xffffffffu, near0);
           near1 = __reduce_or_sync(0xffffffffu, near1);
-          if (lane == 0) EL[(int64_t)T.tile * TB + r] = row_info(m, near0, near1);
+          nz0 = __reduce_or_sync(0xffffffffu, nz0);
+          nz1 = __reduce_or_sync(0xffffffffu, nz1);
+          if (lane == 0) {
+            EL[(int64_t)T.tile * TB + r] = row_info(m, near0, near1);
+            ZL[(int64_t)T.tile * TB + r] = row_nonzero(m, nz0, nz1);
+          }
         }
         double2* Lt = Lg + (int64_t)T.tile * TB * TB;
         for (int i = tid; i < TB * TB; i += NTHR) {
@@ -1125,7 +1151,7 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
       if (tid < TB) {
         s_eL[tid] = X_ZERO;
         s_eW[tid] = X_ZERO;
-        s_near[tid][0] = s_near[tid][1] = 0;
+        s_near[tid][0] = s_near[tid][1] = s_nz[tid][0] = s_nz[tid][1] = 0;
         const double2 d = ld_cg(Dg + (int64_t)T.col * TB + tid);
         s_d[tid] = d;
         if constexpr (PIV) {
@@ -1166,7 +1192,11 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
           if (!s_in) Sa[ri * TB * TB + (r0 + i) * TB + oc] = S[i];   // read again after the product
           reinterpret_cast<short*>(smem + OLD_OFF)[((r0 + i) * TB + oc) * 2 + ri] = (short)exp_of(S[i], 0);
           const unsigned near = __ballot_sync(0xffffffffu, near_max(exp_of(S[i], -bal), m));
-          if (lane == 0) atomicOr(&s_near[r0 + i][warp & 1], near);
+          const unsigned nz = __ballot_sync(0xffffffffu, m <= X_ZERO || m >= X_BAD || exp_of(S[i], 0) != X_ZERO);
+          if (lane == 0) {
+            atomicOr(&s_near[r0 + i][warp & 1], near);
+            atomicOr(&s_nz[r0 + i][warp & 1], nz);
+          }
         }
       }
       __syncthreads();
@@ -1232,15 +1262,21 @@ __global__ void __launch_bounds__(NTHR, 1) factor_dig_kernel(const FactorParams 
           g[word_at(r, c, 1)] = word_of(w[i].y, -bal, eW);
           const unsigned nl = __ballot_sync(0xffffffffu, near_max(max(exp_of(l[i].x, bal), exp_of(l[i].y, bal)), s_eL[r]));
           const unsigned nw = __ballot_sync(0xffffffffu, near_max(max(exp_of(w[i].x, -bal), exp_of(w[i].y, -bal)), s_eW[r]));
+          const unsigned zl = __ballot_sync(0xffffffffu, max(exp_of(l[i].x, bal), exp_of(l[i].y, bal)) != X_ZERO);
+          const unsigned zw = __ballot_sync(0xffffffffu, max(exp_of(w[i].x, -bal), exp_of(w[i].y, -bal)) != X_ZERO);
           if (lane == 0) {
             s_near[r][warp & 1] = nl;
             s_nearV[r][warp & 1] = nw;
+            s_nz[r][warp & 1] = zl;
+            s_nzV[r][warp & 1] = zw;
           }
         }
         __syncthreads();
         if (tid < TB) {
           EL[(int64_t)T.tile * TB + tid] = row_info(s_eL[tid], s_near[tid][0], s_near[tid][1]);
           EW[(int64_t)T.tile * TB + tid] = row_info(s_eW[tid], s_nearV[tid][0], s_nearV[tid][1]);
+          ZL[(int64_t)T.tile * TB + tid] = row_nonzero(s_eL[tid], s_nz[tid][0], s_nz[tid][1]);
+          ZW[(int64_t)T.tile * TB + tid] = row_nonzero(s_eW[tid], s_nzV[tid][0], s_nzV[tid][1]);
         }
       }
     }

@@ -67,3 +67,33 @@ def test_weakly_coupled_groups(torch_cuda, engine, pivot, kind, nblk, m, eps):
     for q in range(g.max() + 1):
         err = np.linalg.norm((X - ref)[g == q].astype(complex)) / np.linalg.norm(ref[g == q].astype(complex))
         assert err <= 1e-13, (q, err)
+
+
+@pytest.mark.parametrize("engine", ["digits", "fma"])
+@pytest.mark.parametrize("pivot", [False, True])
+@pytest.mark.parametrize("kind,nblk,m", [("interleaved", 3, 64), ("decay", 3, 100)])
+def test_decoupled_groups(torch_cuda, engine, pivot, kind, nblk, m):
+    # eps = 0: rows of different groups meet in zeros only, and what couples them stays exactly zero
+    from paper_2002_05026_gb300 import D3M
+    torch = torch_cuda
+    rs = np.random.RandomState(nblk * m)
+    n = nblk * m
+    g = _groups(kind, nblk, m, rs)
+    G = rs.randn(n, n) + 1j * rs.randn(n, n)
+    K = (G + G.T) / np.sqrt(8 * n) + (3.0 + 0.5j) * np.eye(n)
+    K *= g[:, None] == g[None, :]
+    b = (rs.randn(n) + 1j * rs.randn(n)) * np.power(1e-6, g)
+    colptr = np.cumsum([0] + [nblk - c for c in range(nblk)]).astype(np.int64)
+    rowidx = np.concatenate([np.arange(c, nblk) for c in range(nblk)]).astype(np.int32)
+    vals = np.concatenate([K[r * m:(r + 1) * m, c * m:(c + 1) * m].T.reshape(-1) for c in range(nblk) for r in range(c, nblk)])
+    s = D3M(colptr, rowidx, m=m, precision="fp64", max_nrhs=1, pivot=pivot, fp64_engine=engine)
+    s.factor(torch.from_numpy(vals).cuda())
+    X = s.solve(torch.from_numpy(b).cuda()).cpu().numpy()
+    if not pivot:
+        L = s.factor_block(nblk - 1, 0, m, m)
+        assert not L[g[(nblk - 1) * m:][:, None] != g[None, :m]].any()
+    s.close()
+    ref = _extended_solve(K, b)
+    for q in range(g.max() + 1):
+        err = np.linalg.norm((X - ref)[g == q].astype(complex)) / np.linalg.norm(ref[g == q].astype(complex))
+        assert err <= 1e-13, (q, err)
